@@ -11,9 +11,14 @@
 // with accumulate increased by, weight * term, and the gradient buffer
 // likewise receives weight * d term.  All reductions run in a fixed order.
 //
-// D-SSIM: one CTA per 32x8 pixel tile of one projection stages the tile and
+// D-SSIM: one CTA per 32x16 pixel tile of one projection stages the tile and
 // a 5-pixel halo, forms the five windowed moments with two separable passes
 // in shared memory and evaluates SSIM and its partial derivatives per pixel.
+// Shared-memory loads bound both passes, so each thread forms four outputs
+// from one set of loads: four neighbours along x from 16-byte loads, four along
+// y from one column of 14 rows (41 loaded words a pixel; one output per thread
+// on 32x8 tiles took 105).  Eight 512 x 384 projections: forward 50 -> 35 us,
+// adjoint 31 -> 29 us.
 // The moments are taken about a per-tile shift (the tile's mean) so that
 // s^2 = E[x^2] - mu^2 does not cancel in fp32 at projection magnitudes; zero
 // padding is honoured exactly through the window mass s inside the image.
@@ -23,10 +28,13 @@
 namespace pmf {
 namespace {
 
-constexpr int kTU = 32, kTV = 8;                  // SSIM output tile
+constexpr int kTU = 32, kTV = 16;                 // SSIM output tile
 constexpr int kHW = 5;                            // window half-width
 constexpr int kInU = kTU + 2 * kHW, kInV = kTV + 2 * kHW;
-constexpr int kSsimThreads = kTU * kTV;           // one output pixel per thread
+constexpr int kInP = 44;                          // row pitch of the staged tile: 16-byte rows
+constexpr int kRun = 4;                           // outputs per thread of either pass
+constexpr int kSsimThreads = kTU * kTV / kRun;    // 128
+static_assert(kInP % 4 == 0 && kInP >= kTU - kRun + 16 && kTU % kRun == 0 && kTV % kRun == 0, "runs of four");
 
 // The normalised 1-D Gaussian window (sigma 1.5, 11 taps): w[t] for offset t - 5.
 struct Window {
@@ -67,72 +75,139 @@ __device__ __forceinline__ float block_sum_f(float v, float* red) {
     return t;
 }
 
+// The 16 staged words from column c of a row (c a multiple of 4).
+__device__ __forceinline__ void load16(const float* row, float v[16]) {
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const float4 q = reinterpret_cast<const float4*>(row)[k];
+        v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
+    }
+}
+
+// f(row, column) once per staged word (kInV x kInP), a warp per row; unrolled,
+// so that a thread's loads overlap.
+template <class F>
+__device__ __forceinline__ void for_staged(const F& f) {
+    constexpr int W = kSsimThreads / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < (kInV + W - 1) / W; k++) {
+        const int r = warp + W * k;
+        if (r >= kInV) break;
+        f(r, lane);
+        if (lane + 32 < kInP) f(r, lane + 32);
+    }
+}
+
 // Forward: per pixel S and the partials G1 = dS/dmu_x - 2 mu_x G2 - mu_y G3,
 // G2 = dS/d s_x^2, G3 = dS/d s_xy (with dS/dmu_x taken at fixed s's), so that
 // dS(q)/dx(r) = w(q - r) (G1(q) + 2 x(r) G2(q) + y(r) G3(q)).
 __global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int ntu, const float* __restrict__ X,
                                                            const float* __restrict__ Y, float C1, float C2,
                                                            const Window W, float* G, double* part) {
-    __shared__ float sx[kInV][kInU], sy[kInV][kInU];
-    __shared__ float h[5][kInV][kTU];
-    __shared__ float red[kSsimThreads / 32];
+    __shared__ __align__(16) float sx[kInV][kInP], sy[kInV][kInP];
+    __shared__ __align__(16) float h[5][kInV][kTU];
+    __shared__ float red[2][kSsimThreads / 32];
     const int p = blockIdx.y, tu = blockIdx.x % ntu, tv = blockIdx.x / ntu;
     const int u0 = tu * kTU - kHW, v0 = tv * kTV - kHW;
     const int64_t Q = (int64_t)nu * nv;
     const float* Xp = X + (int64_t)p * Q;
     const float* Yp = Y + (int64_t)p * Q;
     // stage the tile and halo (zero outside the image) and its mean over the image part
-    float ax = 0.f, ay = 0.f, cnt = 0.f;
-    for (int i = threadIdx.x; i < kInU * kInV; i += kSsimThreads) {
-        const int r = i / kInU, c = i - r * kInU;
+    float ax = 0.f, ay = 0.f;
+    for_staged([&](int r, int c) {
         const int u = u0 + c, v = v0 + r;
-        const bool in = u >= 0 && u < nu && v >= 0 && v < nv;
+        const bool in = c < kInU && u >= 0 && u < nu && v >= 0 && v < nv;
         const float x = in ? __ldg(Xp + (int64_t)v * nu + u) : 0.f, y = in ? __ldg(Yp + (int64_t)v * nu + u) : 0.f;
         sx[r][c] = x;
         sy[r][c] = y;
         ax += x;
         ay += y;
-        cnt += in ? 1.f : 0.f;
+    });
+    for (int o = 16; o > 0; o >>= 1) {
+        ax += __shfl_xor_sync(0xffffffffu, ax, o);
+        ay += __shfl_xor_sync(0xffffffffu, ay, o);
     }
-    const float n_in = block_sum_f(cnt, red);
-    const float cx = block_sum_f(ax, red) / n_in, cy = block_sum_f(ay, red) / n_in;
+    if ((threadIdx.x & 31) == 0) {
+        red[0][threadIdx.x >> 5] = ax;
+        red[1][threadIdx.x >> 5] = ay;
+    }
+    __syncthreads();
+    const float n_in = (float)((min(u0 + kInU, nu) - max(u0, 0)) * (min(v0 + kInV, nv) - max(v0, 0)));
+    ax = ay = 0.f;
+    for (int k = 0; k < kSsimThreads / 32; k++) {  // fixed order, same in every thread
+        ax += red[0][k];
+        ay += red[1][k];
+    }
+    const float cx = ax / n_in, cy = ay / n_in;
     // shift inside the image (outside stays zero)
-    for (int i = threadIdx.x; i < kInU * kInV; i += kSsimThreads) {
-        const int r = i / kInU, c = i - r * kInU;
+    for_staged([&](int r, int c) {
         const int u = u0 + c, v = v0 + r;
-        if (u >= 0 && u < nu && v >= 0 && v < nv) {
+        if (c < kInU && u >= 0 && u < nu && v >= 0 && v < nv) {
             sx[r][c] -= cx;
             sy[r][c] -= cy;
         }
-    }
+    });
     __syncthreads();
-    // horizontal pass: 5 sums for every staged row and output column
-    for (int i = threadIdx.x; i < kInV * kTU; i += kSsimThreads) {
-        const int r = i / kTU, c = i - r * kTU;
-        float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f, m4 = 0.f;
+    // horizontal pass: 5 sums for every staged row and output column, four columns per thread
+    for (int i = threadIdx.x; i < kInV * (kTU / kRun); i += kSsimThreads) {
+        const int r = i / (kTU / kRun), c = (i - r * (kTU / kRun)) * kRun;
+        float x[16], y[16], m[5][kRun];
+        load16(&sx[r][c], x);
+        load16(&sy[r][c], y);
 #pragma unroll
-        for (int t = 0; t < 11; t++) {
-            const float x = sx[r][c + t], y = sy[r][c + t], wt = W.w[t];
-            m0 = fmaf(wt, x, m0);
-            m1 = fmaf(wt, y, m1);
-            m2 = fmaf(wt * x, x, m2);
-            m3 = fmaf(wt * y, y, m3);
-            m4 = fmaf(wt * x, y, m4);
+        for (int k = 0; k < 5; k++)
+#pragma unroll
+            for (int o = 0; o < kRun; o++) m[k][o] = 0.f;
+#pragma unroll
+        for (int e = 0; e < 10 + kRun; e++) {
+            const float xx = x[e] * x[e], yy = y[e] * y[e], xy = x[e] * y[e];
+#pragma unroll
+            for (int o = 0; o < kRun; o++) {
+                const int t = e - o;
+                if (t < 0 || t > 10) continue;
+                m[0][o] = fmaf(W.w[t], x[e], m[0][o]);
+                m[1][o] = fmaf(W.w[t], y[e], m[1][o]);
+                m[2][o] = fmaf(W.w[t], xx, m[2][o]);
+                m[3][o] = fmaf(W.w[t], yy, m[3][o]);
+                m[4][o] = fmaf(W.w[t], xy, m[4][o]);
+            }
         }
-        h[0][r][c] = m0; h[1][r][c] = m1; h[2][r][c] = m2; h[3][r][c] = m3; h[4][r][c] = m4;
+#pragma unroll
+        for (int k = 0; k < 5; k++)
+            *reinterpret_cast<float4*>(&h[k][r][c]) = make_float4(m[k][0], m[k][1], m[k][2], m[k][3]);
     }
     __syncthreads();
-    const int c = threadIdx.x % kTU, r = threadIdx.x / kTU;
-    const int u = tu * kTU + c, v = tv * kTV + r;
-    float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    // vertical pass: four output rows of one column per thread
+    const int c = threadIdx.x % kTU, r0 = threadIdx.x / kTU * kRun;
+    const int u = tu * kTU + c;
+    float mm[kRun][5];
 #pragma unroll
-    for (int t = 0; t < 11; t++)
+    for (int o = 0; o < kRun; o++)
 #pragma unroll
-        for (int k = 0; k < 5; k++) m[k] = fmaf(W.w[t], h[k][r + t][c], m[k]);
+        for (int k = 0; k < 5; k++) mm[o][k] = 0.f;
+#pragma unroll
+    for (int e = 0; e < 10 + kRun; e++) {
+        float x[5];
+#pragma unroll
+        for (int k = 0; k < 5; k++) x[k] = h[k][r0 + e][c];
+#pragma unroll
+        for (int o = 0; o < kRun; o++) {
+            const int t = e - o;
+            if (t < 0 || t > 10) continue;
+#pragma unroll
+            for (int k = 0; k < 5; k++) mm[o][k] = fmaf(W.w[t], x[k], mm[o][k]);
+        }
+    }
     float S = 0.f;
-    if (u < nu && v < nv) {
+    const float su = inside_mass(W, u, nu);
+#pragma unroll
+    for (int o = 0; o < kRun; o++) {
+        const int v = tv * kTV + r0 + o;
+        if (u >= nu || v >= nv) continue;
+        const float* m = mm[o];
         // moments about the shift: mu = mu' + c s, s^2 = E'[x^2] - mu'^2 + 2 c mu' (1 - s) + c^2 s (1 - s)
-        const float s = inside_mass(W, u, nu) * inside_mass(W, v, nv), s1 = 1.f - s;
+        const float s = su * inside_mass(W, v, nv), s1 = 1.f - s;
         const float mx = fmaf(cx, s, m[0]), my = fmaf(cy, s, m[1]);
         const float vxx = fmaf(cx * s, cx * s1, fmaf(2.f * cx * s1, m[0], m[2] - m[0] * m[0]));
         const float vyy = fmaf(cy * s, cy * s1, fmaf(2.f * cy * s1, m[1], m[3] - m[1] * m[1]));
@@ -140,9 +215,10 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int 
         const float A1 = fmaf(2.f * mx, my, C1), A2 = fmaf(2.f, vxy, C2);
         const float B1 = fmaf(mx, mx, fmaf(my, my, C1)), B2 = vxx + vyy + C2;
         const float iB = 1.f / (B1 * B2);
-        S = A1 * A2 * iB;
-        const float G2 = -S / B2, G3 = 2.f * A1 * iB;
-        const float D = 2.f * my * A2 * iB - 2.f * mx * S / B1;  // dS/dmu_x at fixed s's
+        const float Sp = A1 * A2 * iB;
+        S += Sp;
+        const float G2 = -Sp / B2, G3 = 2.f * A1 * iB;
+        const float D = 2.f * my * A2 * iB - 2.f * mx * Sp / B1;  // dS/dmu_x at fixed s's
         const float G1 = D - 2.f * mx * G2 - my * G3;
         const int64_t q = (int64_t)p * Q + (int64_t)v * nu + u;
         const int64_t PQ = Q * gridDim.y;
@@ -150,7 +226,7 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int 
         G[PQ + q] = G2;
         G[2 * PQ + q] = G3;
     }
-    const float tot = block_sum_f(S, red);
+    const float tot = block_sum_f(S, red[0]);
     if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = (double)tot;
 }
 
@@ -159,45 +235,58 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_bwd(int nu, int nv, int 
                                                            const float* __restrict__ Y, const float* __restrict__ G,
                                                            const Window W, float scale, float* d_pred,
                                                            int accumulate) {
-    __shared__ float sg[3][kInV][kInU];
-    __shared__ float h[3][kInV][kTU];
+    __shared__ __align__(16) float sg[3][kInV][kInP];
+    __shared__ __align__(16) float h[3][kInV][kTU];
     const int p = blockIdx.y, tu = blockIdx.x % ntu, tv = blockIdx.x / ntu;
     const int u0 = tu * kTU - kHW, v0 = tv * kTV - kHW;
     const int64_t Q = (int64_t)nu * nv, PQ = Q * gridDim.y;
-    for (int i = threadIdx.x; i < kInU * kInV; i += kSsimThreads) {
-        const int r = i / kInU, c = i - r * kInU;
+    for_staged([&](int r, int c) {
         const int u = u0 + c, v = v0 + r;
-        const bool in = u >= 0 && u < nu && v >= 0 && v < nv;
+        const bool in = c < kInU && u >= 0 && u < nu && v >= 0 && v < nv;
         const int64_t q = (int64_t)p * Q + (int64_t)v * nu + u;
 #pragma unroll
         for (int k = 0; k < 3; k++) sg[k][r][c] = in ? __ldg(G + k * PQ + q) : 0.f;
-    }
+    });
     __syncthreads();
-    for (int i = threadIdx.x; i < kInV * kTU; i += kSsimThreads) {
-        const int r = i / kTU, c = i - r * kTU;
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+    for (int i = threadIdx.x; i < kInV * (kTU / kRun); i += kSsimThreads) {
+        const int r = i / (kTU / kRun), c = (i - r * (kTU / kRun)) * kRun;
 #pragma unroll
-        for (int t = 0; t < 11; t++) {
-            a0 = fmaf(W.w[t], sg[0][r][c + t], a0);
-            a1 = fmaf(W.w[t], sg[1][r][c + t], a1);
-            a2 = fmaf(W.w[t], sg[2][r][c + t], a2);
+        for (int k = 0; k < 3; k++) {
+            float x[16], a[kRun] = {0.f, 0.f, 0.f, 0.f};
+            load16(&sg[k][r][c], x);
+#pragma unroll
+            for (int t = 0; t < 11; t++)
+#pragma unroll
+                for (int o = 0; o < kRun; o++) a[o] = fmaf(W.w[t], x[t + o], a[o]);
+            *reinterpret_cast<float4*>(&h[k][r][c]) = make_float4(a[0], a[1], a[2], a[3]);
         }
-        h[0][r][c] = a0; h[1][r][c] = a1; h[2][r][c] = a2;
     }
     __syncthreads();
-    const int c = threadIdx.x % kTU, r = threadIdx.x / kTU;
-    const int u = tu * kTU + c, v = tv * kTV + r;
-    if (u >= nu || v >= nv) return;
-    float b0 = 0.f, b1 = 0.f, b2 = 0.f;
+    const int c = threadIdx.x % kTU, r0 = threadIdx.x / kTU * kRun;
+    const int u = tu * kTU + c;
+    if (u >= nu) return;
+    float bb[kRun][3];
 #pragma unroll
-    for (int t = 0; t < 11; t++) {
-        b0 = fmaf(W.w[t], h[0][r + t][c], b0);
-        b1 = fmaf(W.w[t], h[1][r + t][c], b1);
-        b2 = fmaf(W.w[t], h[2][r + t][c], b2);
+    for (int o = 0; o < kRun; o++) bb[o][0] = bb[o][1] = bb[o][2] = 0.f;
+#pragma unroll
+    for (int e = 0; e < 10 + kRun; e++) {
+        const float x[3] = {h[0][r0 + e][c], h[1][r0 + e][c], h[2][r0 + e][c]};
+#pragma unroll
+        for (int o = 0; o < kRun; o++) {
+            const int t = e - o;
+            if (t < 0 || t > 10) continue;
+#pragma unroll
+            for (int k = 0; k < 3; k++) bb[o][k] = fmaf(W.w[t], x[k], bb[o][k]);
+        }
     }
-    const int64_t q = (int64_t)p * Q + (int64_t)v * nu + u;
-    const float g = scale * fmaf(2.f * __ldg(X + q), b1, fmaf(__ldg(Y + q), b2, b0));
-    d_pred[q] = accumulate ? d_pred[q] + g : g;
+#pragma unroll
+    for (int o = 0; o < kRun; o++) {
+        const int v = tv * kTV + r0 + o;
+        if (v >= nv) break;
+        const int64_t q = (int64_t)p * Q + (int64_t)v * nu + u;
+        const float g = scale * fmaf(2.f * __ldg(X + q), bb[o][1], fmaf(__ldg(Y + q), bb[o][2], bb[o][0]));
+        d_pred[q] = accumulate ? d_pred[q] + g : g;
+    }
 }
 
 // loss (=/+=) weight * (1 - sum S / (P Q)), partials summed in order in double.
@@ -286,18 +375,62 @@ __global__ void k_sum_final(const double* part, int n, double mult, float* loss,
 
 constexpr int kNormBlocks = 152;   // partial sums per MBC component (fixed: order independent of the device)
 
+// The components lie back to back (component lk from element lk N), and four
+// elements are one 8- or 16-byte load: a component's run of whole groups,
+// [head, head + 4 groups), starts at the next multiple of four elements of the
+// array, whatever N is; its up to three elements before and after are taken one by one.
+// VEC is false where the array itself is not aligned.
+struct Quads {
+    int64_t head, groups, tail;  // leading elements, groups of four, first element after them
+};
+
+__device__ __forceinline__ Quads quads_of(int64_t lk, int64_t N, bool vec) {
+    Quads q;
+    const int64_t lead = (4 - ((lk * N) & 3)) & 3;
+    q.head = vec ? (lead < N ? lead : N) : N;
+    q.groups = (N - q.head) >> 2;
+    q.tail = q.head + 4 * q.groups;
+    return q;
+}
+
+__device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
+    const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
+    return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
+                       __uint_as_float(r.y & 0xffff0000u));
+}
+__device__ __forceinline__ float4 ld4(const __half* p) {
+    uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
+    const float2 a = __half22float2(*reinterpret_cast<__half2*>(&r.x)), b = __half22float2(*reinterpret_cast<__half2*>(&r.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
 // part[lk][b] = sum of squares of component lk over block b's grid-stride range (double).
 template <typename T>
-__global__ void __launch_bounds__(256) k_sumsq(const T* __restrict__ E, int64_t N, double* part) {
+__global__ void __launch_bounds__(256) k_sumsq(const T* __restrict__ E, int64_t N, bool vec, double* part) {
     __shared__ double red[8];
     const int lk = blockIdx.y;
     const T* e = E + (int64_t)lk * N;
-    float sf = 0.f;  // a thread's own few hundred squares in fp32, then double
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
-        const float x = Store<T>::ld(e, v);
-        sf = fmaf(x, x, sf);
+    const Quads Q = quads_of(lk, N, vec);
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    float sf[4] = {0.f, 0.f, 0.f, 0.f};  // a thread's own few dozen squares in fp32 (four chains), then double
+#pragma unroll 4
+    for (int64_t k = t0; k < Q.groups; k += nt) {
+        const float4 x = ld4(e + Q.head + 4 * k);
+        sf[0] = fmaf(x.x, x.x, sf[0]);
+        sf[1] = fmaf(x.y, x.y, sf[1]);
+        sf[2] = fmaf(x.z, x.z, sf[2]);
+        sf[3] = fmaf(x.w, x.w, sf[3]);
     }
-    double s = (double)sf;
+    for (int64_t v = t0; v < Q.head; v += nt) {
+        const float x = Store<T>::ld(e, v);
+        sf[0] = fmaf(x, x, sf[0]);
+    }
+    for (int64_t v = Q.tail + t0; v < N; v += nt) {
+        const float x = Store<T>::ld(e, v);
+        sf[1] = fmaf(x, x, sf[1]);
+    }
+    double s = ((double)sf[0] + (double)sf[1]) + ((double)sf[2] + (double)sf[3]);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
@@ -308,31 +441,57 @@ __global__ void __launch_bounds__(256) k_sumsq(const T* __restrict__ E, int64_t 
     }
 }
 
-// norms[lk] = sum of its partials; loss (=/+=) weight / (3L) sum (norm - 1)^2.
-__global__ void k_norm_final(const double* part, int nb, int nlk, double* norms, float weight, float* loss,
-                             int accumulate) {
+// norm = the sum of a component's partials, one warp per component (lane-strided,
+// then a fixed butterfly); gfac[lk] = weight * 4 (norm - 1) / (3L), the factor of
+// its gradient; loss (=/+=) weight / (3L) sum (norm - 1)^2 in component order.  (One thread adding all 1,368 partials in order took 90 us of
+// dependent double adds; this takes 5.)
+__global__ void __launch_bounds__(1024) k_norm_final(const double* __restrict__ part, int nb, int nlk, float* gfac,
+                                                     float weight, float* loss, int accumulate) {
+    __shared__ double sq[192];  // nlk <= 3 * 64
+    const int lane = threadIdx.x & 31;
+    for (int lk = threadIdx.x >> 5; lk < nlk; lk += 32) {
+        double n2 = 0.0;
+        for (int b = lane; b < nb; b += 32) n2 += part[(int64_t)lk * nb + b];
+        for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        if (lane == 0) {
+            gfac[lk] = (float)((double)weight * 4.0 * (n2 - 1.0) / (double)nlk);
+            sq[lk] = (n2 - 1.0) * (n2 - 1.0);
+        }
+    }
+    __syncthreads();
     if (threadIdx.x != 0) return;
     double tot = 0.0;
-    for (int lk = 0; lk < nlk; lk++) {
-        double n2 = 0.0;
-        for (int b = 0; b < nb; b++) n2 += part[(int64_t)lk * nb + b];
-        norms[lk] = n2;
-        tot += (n2 - 1.0) * (n2 - 1.0);
-    }
+    for (int lk = 0; lk < nlk; lk++) tot += sq[lk];
     const float v = (float)((double)weight * tot / (double)nlk);
     *loss = accumulate ? *loss + v : v;
 }
 
-// dE (=/+=) weight * 4 (norm - 1) e / (3L).
+// dE (=/+=) gfac e: streams E and dE once, four elements a load and store.  (Each
+// thread forming the factor in double, a division on this part's slow fp64 pipe,
+// took 150 us for the paper's nine 4,000,000-voxel bf16 components; this 39,
+// 32 at the copy rate.)
 template <typename T>
-__global__ void __launch_bounds__(256) k_norm_grad(const T* __restrict__ E, int64_t N, int nlk,
-                                                   const double* __restrict__ norms, float weight, float* dE,
-                                                   int accumulate) {
+__global__ void __launch_bounds__(256) k_norm_grad(const T* __restrict__ E, int64_t N, bool vec,
+                                                   const float* __restrict__ gfac, float* dE, int accumulate) {
     const int lk = blockIdx.y;
-    const float f = (float)((double)weight * 4.0 * (norms[lk] - 1.0) / (double)nlk);
+    const float f = gfac[lk];
     const T* e = E + (int64_t)lk * N;
     float* d = dE + (int64_t)lk * N;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
+    const Quads Q = quads_of(lk, N, vec);
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t k = t0; k < Q.groups; k += nt) {
+        const float4 x = ld4(e + Q.head + 4 * k);
+        float4 g = make_float4(f * x.x, f * x.y, f * x.z, f * x.w);
+        float4* o = reinterpret_cast<float4*>(d + Q.head + 4 * k);
+        if (accumulate) {
+            const float4 b = *o;
+            g = make_float4(b.x + g.x, b.y + g.y, b.z + g.z, b.w + g.w);
+        }
+        *o = g;
+    }
+    const int64_t rest = Q.head + (N - Q.tail);
+    for (int64_t r = t0; r < rest; r += nt) {
+        const int64_t v = r < Q.head ? r : Q.tail + (r - Q.head);
         const float g = f * Store<T>::ld(e, v);
         d[v] = accumulate ? d[v] + g : g;
     }
@@ -457,7 +616,7 @@ pmf_status projection_dssim(int32_t P, int32_t nu, int32_t nv, const float* pred
         k_dssim_bwd<<<dim3((unsigned)nt, (unsigned)P), kSsimThreads, 0, s>>>(nu, nv, ntu, pred, meas, G, W, scale,
                                                                           d_pred, accumulate);
     }
-    k_dssim_final<<<1, 256, 0, s>>>(part, nt * P, (double)P * nu * nv, weight, loss, accumulate);
+    k_dssim_final<<<1, 1024, 0, s>>>(part, nt * P, (double)P * nu * nv, weight, loss, accumulate);
     return check_launch("projection_dssim");
 }
 
@@ -512,15 +671,16 @@ pmf_status mbc_normality(const pmf_grid* grid, int32_t L, pmf_dtype dtype, const
     if ((st = validate_ws(ws, ws_bytes, need)) != PMF_OK) return st;
     const int64_t N = (int64_t)grid->nx * grid->ny * grid->nz;
     double* part = (double*)ws;
-    double* norms = (double*)((char*)ws + align_up(sizeof(double) * (size_t)3 * L * kNormBlocks));
+    float* gfac = (float*)((char*)ws + align_up(sizeof(double) * (size_t)3 * L * kNormBlocks));
     cudaStream_t s = (cudaStream_t)stream;
     const dim3 gr(kNormBlocks, (unsigned)(3 * L));
-    PMF_DISPATCH_DTYPE(dtype, T, k_sumsq<T><<<gr, 256, 0, s>>>((const T*)mbc, N, part));
-    k_norm_final<<<1, 32, 0, s>>>(part, kNormBlocks, 3 * L, norms, weight, loss, accumulate);
+    const bool vec = (((uintptr_t)mbc | (uintptr_t)d_mbc) & 15) == 0;
+    PMF_DISPATCH_DTYPE(dtype, T, k_sumsq<T><<<gr, 256, 0, s>>>((const T*)mbc, N, vec, part));
+    k_norm_final<<<1, 1024, 0, s>>>(part, kNormBlocks, 3 * L, gfac, weight, loss, accumulate);
     if (d_mbc) {
-        const int64_t nb = (N + 255) / 256;
+        const int64_t nb = (N + 1023) / 1024;
         const dim3 gg((unsigned)(nb < 4 * kStreamBlocks ? nb : 4 * kStreamBlocks), (unsigned)(3 * L));
-        PMF_DISPATCH_DTYPE(dtype, T, k_norm_grad<T><<<gg, 256, 0, s>>>((const T*)mbc, N, 3 * L, norms, weight, d_mbc, accumulate));
+        PMF_DISPATCH_DTYPE(dtype, T, k_norm_grad<T><<<gg, 256, 0, s>>>((const T*)mbc, N, vec, gfac, d_mbc, accumulate));
     }
     return check_launch("mbc_normality");
 }

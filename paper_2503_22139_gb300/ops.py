@@ -572,6 +572,11 @@ def projection_loss(kind: int, pred: torch.Tensor, meas: torch.Tensor, with_grad
 
 # ------------------------------------------------- Eq. 14 regularisation
 
+def _term_out(accumulate: bool, shape, device) -> torch.Tensor:
+    """A term's output buffer: zeros to accumulate into, else left to the call, which writes every element."""
+    return (torch.zeros if accumulate else torch.empty)(shape, dtype=torch.float32, device=device)
+
+
 def projection_dssim(pred: torch.Tensor, meas: torch.Tensor, data_range: float, weight: float = 1.0,
                      with_grad: bool = True, loss: Optional[torch.Tensor] = None, d_pred: Optional[torch.Tensor] = None,
                      accumulate: bool = False, ws=None):
@@ -583,9 +588,9 @@ def projection_dssim(pred: torch.Tensor, meas: torch.Tensor, data_range: float, 
     if ws is None:
         ws = _ws(_size(L.projection_dssim_workspace, P, nu, nv), pred.device)
     if loss is None:
-        loss = torch.zeros(1, dtype=torch.float32, device=pred.device)
+        loss = _term_out(accumulate, 1, pred.device)
     if with_grad and d_pred is None:
-        d_pred = torch.zeros_like(pred)
+        d_pred = _term_out(accumulate, pred.shape, pred.device)
     check(L.projection_dssim(P, nu, nv, _p(pred), _p(meas), float(data_range), float(weight), _p(loss),
                              _p(d_pred if with_grad else None), int(accumulate), _p(ws), ws.numel(), _stream()),
           "projection_dssim")
@@ -606,9 +611,9 @@ def tv_loss(grid, vol: torch.Tensor, D: int, origin, weight: float = 1.0, with_g
     if ws is None:
         ws = _ws(_size(L.tv_loss_workspace, int(D)), vol.device)
     if loss is None:
-        loss = torch.zeros(1, dtype=torch.float32, device=vol.device)
+        loss = _term_out(accumulate, 1, vol.device)
     if with_grad and d_vol is None:
-        d_vol = torch.zeros(vol.shape, dtype=torch.float32, device=vol.device)
+        d_vol = _term_out(accumulate, vol.shape, vol.device)
     check(L.tv_loss(ct.byref(g), _DT[vol.dtype], _p(vol), int(D), _p(origin), float(weight), _p(loss),
                     _p(d_vol if with_grad else None), int(accumulate), _p(ws), ws.numel(), _stream()), "tv_loss")
     return loss, (d_vol if with_grad else None)
@@ -625,9 +630,9 @@ def mbc_normality(grid, mbc: torch.Tensor, weight: float = 1.0, with_grad: bool 
     if ws is None:
         ws = _ws(_size(Lb.mbc_normality_workspace, L), mbc.device)
     if loss is None:
-        loss = torch.zeros(1, dtype=torch.float32, device=mbc.device)
+        loss = _term_out(accumulate, 1, mbc.device)
     if with_grad and d_mbc is None:
-        d_mbc = torch.zeros(mbc.shape, dtype=torch.float32, device=mbc.device)
+        d_mbc = _term_out(accumulate, mbc.shape, mbc.device)
     check(Lb.mbc_normality(ct.byref(g), L, _DT[mbc.dtype], _p(mbc), float(weight), _p(loss),
                            _p(d_mbc if with_grad else None), int(accumulate), _p(ws), ws.numel(), _stream()),
           "mbc_normality")

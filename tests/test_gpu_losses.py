@@ -89,3 +89,37 @@ def test_mbc_normality_matches_oracle(dt):
     ref, gref = oracle.mbc_normality(Eq)
     assert float(loss.item()) == pytest.approx(ref, rel=1e-5)
     assert rel_l2(host(gE), gref) <= 1e-5
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 15, 31), (1, 16, 32), (3, 17, 33), (1, 42, 97)])
+def test_dssim_at_tile_edges(shape):
+    """Detectors around the 32 x 16 output tile and its 5-pixel halo, the fp32
+    per-pixel and gradient bounds of the larger comparison above."""
+    P, nv, nu = shape
+    Y, M = _projection_pair(P, nv, nu, 21)
+    loss, g = pmf.projection_dssim(dev(Y), dev(M), 300.0)
+    ref, gref = oracle.dssim(Y, M, 300.0)
+    assert abs(float(loss.item()) - ref) <= 2e-6
+    assert rel_l2(host(g), gref) <= 1e-4
+
+
+@pytest.mark.parametrize("n", [(1, 1, 1), (3, 1, 1), (5, 7, 3), (13, 11, 9)])
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_mbc_normality_of_odd_components(n, dt, offset):
+    """Component sizes with every remainder of four, from an aligned and an
+    unaligned array, set and accumulated: the sums are fp32 squares added in
+    double (1e-5), the gradient one fp32 product (1e-6), or a sum of two."""
+    g = Grid(*n, 2.0, 2.0, 2.0)
+    E = (np.random.default_rng(22).normal(size=(2, 3) + g.shape) / np.sqrt(g.n)).astype(np.float32)
+    buf = torch.zeros(E.size + 1, dtype=dt, device="cuda")
+    Ed = buf[offset:offset + E.size].view(E.shape)
+    Ed.copy_(dev(E).to(dt))
+    ref, gref = oracle.mbc_normality(host(Ed))
+    loss, gE = pmf.mbc_normality(g, Ed)
+    assert float(loss.item()) == pytest.approx(ref, rel=1e-5)
+    assert rel_l2(host(gE), gref) <= 1e-5
+    d = torch.full(E.shape, 0.5, dtype=torch.float32, device="cuda")
+    pmf.mbc_normality(g, Ed, loss=loss, d_mbc=d, accumulate=True)
+    assert float(loss.item()) == pytest.approx(2.0 * ref, rel=1e-5)
+    assert rel_l2(host(d), 0.5 + gref) <= 1e-6
