@@ -87,21 +87,93 @@ __device__ __forceinline__ void voxel_ijk(int64_t v, const GridD& g, int& i, int
 
 // ----------------------------------------------------------- combine
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_combine(GridD g, int L, int P, const T* __restrict__ E,
-                                                      const float* __restrict__ w, T* __restrict__ D) {
-    const int64_t N = g.n;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
-        float e[kMaxL][3];
-        for (int l = 0; l < L; l++)
+// V consecutive stored values as floats (V = 4: one 8- or 16-byte load).
+template <int V>
+__device__ __forceinline__ void ld_run(const float* p, float o[V]) {
+    if constexpr (V == 4) {
+        const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+        o[0] = q.x; o[1] = q.y; o[2] = q.z; o[3] = q.w;
+    } else if constexpr (V == 2) {
+        const float2 q = __ldg(reinterpret_cast<const float2*>(p));
+        o[0] = q.x; o[1] = q.y;
+    } else {
+        o[0] = __ldg(p);
+    }
+}
+template <int V, typename T>
+__device__ __forceinline__ void ld_run(const T* p, float o[V]) {
+    if constexpr (V == 1) {
+        o[0] = Store<T>::ld(p, 0);
+    } else {
+        struct alignas(2 * V) Run { T v[V]; };
+        unsigned r[(V + 1) / 2];
+        if constexpr (V == 4) {
+            const uint2 q = __ldg(reinterpret_cast<const uint2*>(p));
+            r[0] = q.x; r[1] = q.y;
+        } else {
+            r[0] = __ldg(reinterpret_cast<const unsigned*>(p));
+        }
+        const Run& q = reinterpret_cast<const Run&>(r);
 #pragma unroll
-            for (int k = 0; k < 3; k++) e[l][k] = Store<T>::ld(E, ((int64_t)l * 3 + k) * N + v);
+        for (int i = 0; i < V; i++) o[i] = (float)q.v[i];
+    }
+}
+template <int V>
+__device__ __forceinline__ void st_run(float* p, const float v[V]) {
+    if constexpr (V == 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (V == 2) *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    else p[0] = v[0];
+}
+template <int V, typename T>
+__device__ __forceinline__ void st_run(T* p, const float v[V]) {
+    if constexpr (V == 1) {
+        Store<T>::st(p, 0, v[0]);
+    } else {
+        struct alignas(2 * V) Run { T v[V]; } r;
+#pragma unroll
+        for (int i = 0; i < V; i++) Store<T>::st(r.v, i, v[i]);
+        *reinterpret_cast<Run*>(p) = r;
+    }
+}
+
+// Whether V-voxel runs of [..][N] arrays start on run boundaries.
+template <int V>
+bool runs_aligned(int64_t N, const void* a, const void* b) {
+    return N % V == 0 && ((((uintptr_t)a) | ((uintptr_t)b)) & 15) == 0;
+}
+
+// Streams E once and D once per view, LL levels (0: the runtime L) of V
+// consecutive voxels in registers.  Bandwidth bound: at the paper grid, three
+// levels and one fp32 view, 192 MB take 28 us at the copy rate; one voxel per
+// thread with the level count at run time took 60 us, four per thread 27.
+template <typename T, int LL, int V>
+__global__ void __launch_bounds__(kThreads) k_combine(GridD g, int Lr, int P, const T* __restrict__ E,
+                                                      const float* __restrict__ w, T* __restrict__ D) {
+    constexpr int M = LL ? LL : kMaxL;
+    const int L = LL ? LL : Lr;
+    const int64_t N = g.n;
+    for (int64_t v = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); v < N;
+         v += V * (int64_t)gridDim.x * blockDim.x) {
+        float e[M][3][V];
+#pragma unroll
+        for (int l = 0; l < M; l++)
+#pragma unroll
+            for (int k = 0; k < 3; k++)
+                if (l < L) ld_run<V>(E + ((int64_t)l * 3 + k) * N + v, e[l][k]);
         for (int p = 0; p < P; p++) {
 #pragma unroll
             for (int k = 0; k < 3; k++) {
-                float acc = 0.f;
-                for (int l = 0; l < L; l++) acc = fmaf(__ldg(w + (p * L + l) * 3 + k), e[l][k], acc);
-                Store<T>::st(D, ((int64_t)p * 3 + k) * N + v, acc);
+                float acc[V];
+#pragma unroll
+                for (int i = 0; i < V; i++) acc[i] = 0.f;
+#pragma unroll
+                for (int l = 0; l < M; l++)
+                    if (l < L) {
+                        const float c = __ldg(w + (p * L + l) * 3 + k);
+#pragma unroll
+                        for (int i = 0; i < V; i++) acc[i] = fmaf(c, e[l][k][i], acc[i]);
+                    }
+                st_run<V>(D + ((int64_t)p * 3 + k) * N + v, acc);
             }
         }
     }
@@ -163,51 +235,56 @@ __global__ void k_reduce_partials(const float* part, int64_t nout, int nb, float
 
 // --------------------------------------------------------------- warp
 
+// A CTA takes 32 x 8 voxels of kWarpZ planes of one view (a lane its kWarpZ
+// voxels of one column): the voxel's coordinates come from one 32-bit block
+// index, where the flat index cost three 64-bit divisions per voxel, and the
+// loads of a lane's voxels overlap.  At the paper grid, one fp32 view: 43 ->
+// 30 us (80 MB: 12 us at the copy rate).
+constexpr int kWarpZ = 2;
+
+struct WarpTiles {
+    unsigned ntx, nty, ntz;
+    unsigned per_view() const { return ntx * nty * ntz; }
+};
+
+WarpTiles warp_tiles(const GridD& g) {
+    return WarpTiles{(unsigned)((g.nx + 31) / 32), (unsigned)((g.ny + 7) / 8), (unsigned)((g.nz + kWarpZ - 1) / kWarpZ)};
+}
+
+// Views per launch, so that the block index stays below 2^31 (a view has at
+// most n / 2 blocks, on a grid one voxel wide and high).
+int views_per_launch(const WarpTiles& nt) {
+    const int64_t per = (((int64_t)1 << 31) - 1) / nt.per_view();
+    return (int)(per > 0 ? per : 1);
+}
+
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_warp(GridD g, int P, const T* __restrict__ ref, const T* __restrict__ D,
-                                                   T* __restrict__ W) {
-    const int64_t N = g.n, total = N * P;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = t / N, v = t - p * N;
-        int i, j, k;
-        voxel_ijk(v, g, i, j, k);
-        const T* Dp = D + p * 3 * N;
-        const Cell c = make_cell(i, j, k, Store<T>::ld(Dp, v) * g.ivx, Store<T>::ld(Dp, N + v) * g.ivy,
-                                 Store<T>::ld(Dp, 2 * N + v) * g.ivz);
-        Store<T>::st(W, t, trilin_cell(ref, g, c.i0, c.j0, c.k0, c.fx, c.fy, c.fz));
+__global__ void __launch_bounds__(kThreads) k_warp(GridD g, WarpTiles nt, const T* __restrict__ ref,
+                                                   const T* __restrict__ D, T* __restrict__ W) {
+    const unsigned b = blockIdx.x, bz = b / (nt.ntx * nt.nty), r = b - bz * (nt.ntx * nt.nty);
+    const unsigned p = bz / nt.ntz, tz = bz - p * nt.ntz, ty = r / nt.ntx, tx = r - ty * nt.ntx;
+    const int i = (int)(tx * 32 + (threadIdx.x & 31)), j = (int)(ty * 8 + (threadIdx.x >> 5)), k0 = (int)tz * kWarpZ;
+    if (i >= g.nx || j >= g.ny) return;
+    const int64_t N = g.n;
+    const T* Dp = D + (int64_t)p * 3 * N;
+    T* Wp = W + (int64_t)p * N;
+    float d[kWarpZ][3];
+#pragma unroll
+    for (int h = 0; h < kWarpZ; h++) {
+        const int64_t v = ((int64_t)(k0 + h) * g.ny + j) * g.nx + i;
+#pragma unroll
+        for (int c = 0; c < 3; c++) d[h][c] = k0 + h < g.nz ? Store<T>::ld(Dp, c * N + v) : 0.f;
+    }
+#pragma unroll
+    for (int h = 0; h < kWarpZ; h++) {
+        if (k0 + h >= g.nz) break;
+        const int64_t v = ((int64_t)(k0 + h) * g.ny + j) * g.nx + i;
+        const Cell c = make_cell(i, j, k0 + h, d[h][0] * g.ivx, d[h][1] * g.ivy, d[h][2] * g.ivz);
+        Store<T>::st(Wp, v, trilin_cell(ref, g, c.i0, c.j0, c.k0, c.fx, c.fy, c.fz));
     }
 }
 
 __global__ void k_absmax(const float* __restrict__ x, int64_t n, unsigned* out) { absmax_bits(x, n, out); }
-
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_warp_bwd(GridD g, int P, const T* __restrict__ ref,
-                                                       const T* __restrict__ D, const float* __restrict__ dW,
-                                                       float* d_dvf, unsigned long long* acc, const unsigned* maxbits,
-                                                       int accumulate) {
-    const int64_t N = g.n, total = N * P;
-    const int kexp = fixed_exponent(__uint_as_float(*maxbits) * (float)total);
-    const float scale = ldexpf(1.0f, kexp);
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = t / N, v = t - p * N;
-        int i, j, k;
-        voxel_ijk(v, g, i, j, k);
-        const T* Dp = D + p * 3 * N;
-        const Cell c = make_cell(i, j, k, Store<T>::ld(Dp, v) * g.ivx, Store<T>::ld(Dp, N + v) * g.ivy,
-                                 Store<T>::ld(Dp, 2 * N + v) * g.ivz);
-        const float gw = __ldg(dW + t);
-        if (d_dvf) {
-            float gx, gy, gz;
-            trilin_grad(ref, g, c, gx, gy, gz);
-            float* o = d_dvf + p * 3 * N + v;
-            const float r0 = gw * gx * g.ivx, r1 = gw * gy * g.ivy, r2 = gw * gz * g.ivz;
-            o[0] = accumulate ? o[0] + r0 : r0;
-            o[N] = accumulate ? o[N] + r1 : r1;
-            o[2 * N] = accumulate ? o[2 * N] + r2 : r2;
-        }
-        if (gw != 0.f) scatter_cell(acc, g, c, gw, scale);
-    }
-}
 
 // d_ref (=/+=) fixed-point accumulator * 2^-k, k from the same bound.
 __global__ void k_fixed_to_float(const unsigned long long* __restrict__ acc, int64_t n, const unsigned* maxbits,
@@ -826,6 +903,159 @@ __global__ void __launch_bounds__(GeomBwd::THREADS, 2) k_wc_bwd_tile(GridD g, in
     }
 }
 
+// ---------------------------------------------- adjoints of the unfused calls
+
+// The adjoint of warp_volume on k_warp's tiles: the DVF gradient per voxel, and
+// ref's gradient scattered in 64-bit fixed point.  The atomics bind it, and
+// neighbours in x mostly fall in neighbouring cells, where a voxel's four
+// upper-x corners are the next lane's lower-x corners: those are handed over by
+// shuffles and added there first (integer sums: the same bits), so four to eight
+// atomics are left of eight.  At the paper grid, one fp32 view: 78 -> 72 us.  (The
+// fused adjoint's shared-memory box was tried here: with one view per tile its
+// zeroing, staging and flush took 228 us, and 32-bit terms are less exact.)
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_warp_bwd(GridD g, WarpTiles nt, const T* __restrict__ ref,
+                                                       const T* __restrict__ D, const float* __restrict__ dW,
+                                                       float* d_dvf, unsigned long long* acc, const unsigned* maxbits,
+                                                       float bound_mult, int accumulate) {
+    const unsigned b = blockIdx.x, bz = b / (nt.ntx * nt.nty), r = b - bz * (nt.ntx * nt.nty);
+    const unsigned p = bz / nt.ntz, tz = bz - p * nt.ntz, ty = r / nt.ntx, tx = r - ty * nt.ntx;
+    const int lane = threadIdx.x & 31;
+    const int i = (int)tx * 32 + lane, j = (int)(ty * 8 + (threadIdx.x >> 5)), k0 = (int)tz * kWarpZ;
+    if (j >= g.ny) return;  // whole warps
+    const int64_t N = g.n;
+    const T* Dp = D + (int64_t)p * 3 * N;
+    const float* dWp = dW + (int64_t)p * N;
+    const int kexp = fixed_exponent(__uint_as_float(*maxbits) * bound_mult);
+    const float scale = ldexpf(1.0f, kexp);
+    float d[kWarpZ][3], gwv[kWarpZ];
+#pragma unroll
+    for (int h = 0; h < kWarpZ; h++) {
+        const bool in = i < g.nx && k0 + h < g.nz;
+        const int64_t v = ((int64_t)(k0 + h) * g.ny + j) * g.nx + i;
+#pragma unroll
+        for (int c = 0; c < 3; c++) d[h][c] = in ? Store<T>::ld(Dp, c * N + v) : 0.f;
+        gwv[h] = in ? __ldg(dWp + v) : 0.f;
+    }
+#pragma unroll
+    for (int h = 0; h < kWarpZ; h++) {
+        if (k0 + h >= g.nz) break;
+        const int64_t v = ((int64_t)(k0 + h) * g.ny + j) * g.nx + i;
+        const float gw = gwv[h];
+        const Cell c = make_cell(i, j, k0 + h, d[h][0] * g.ivx, d[h][1] * g.ivy, d[h][2] * g.ivz);
+        if (d_dvf && i < g.nx) {
+            float gx, gy, gz;
+            trilin_grad(ref, g, c, gx, gy, gz);
+            float* o = d_dvf + (int64_t)p * 3 * N + v;
+            const float r0 = gw * gx * g.ivx, r1 = gw * gy * g.ivy, r2 = gw * gz * g.ivz;
+            o[0] = accumulate ? o[0] + r0 : r0;
+            o[N] = accumulate ? o[N] + r1 : r1;
+            o[2 * N] = accumulate ? o[2 * N] + r2 : r2;
+        }
+        const bool live = gw != 0.f;  // also false outside the grid
+        // does the lane below (lane - 1) hand its upper-x corners to this lane's lower ones?
+        const int ni = __shfl_up_sync(0xffffffffu, c.i0, 1), nj = __shfl_up_sync(0xffffffffu, c.j0, 1);
+        const int nk = __shfl_up_sync(0xffffffffu, c.k0, 1);
+        const unsigned lives = __ballot_sync(0xffffffffu, live);
+        const bool take = lane > 0 && live && ((lives >> (lane - 1)) & 1u) && ni == c.i0 - 1 && nj == c.j0 && nk == c.k0;
+        const unsigned takes = __ballot_sync(0xffffffffu, take);
+        const bool give = lane < 31 && ((takes >> (lane + 1)) & 1u);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int y = c.j0 + (q & 1), z = c.k0 + (q >> 1);
+            // the weight's products in scatter_cell's order
+            const float wy = (q & 1) ? c.fy : 1.f - c.fy, wz = (q >> 1) ? c.fz : 1.f - c.fz;
+            unsigned long long lo = live ? to_fixed(gw * ((1.f - c.fx) * wy * wz), scale) : 0ull;
+            const unsigned long long hi = live ? to_fixed(gw * (c.fx * wy * wz), scale) : 0ull;
+            const unsigned long long got = __shfl_up_sync(0xffffffffu, hi, 1);
+            if (take) lo += got;
+            if (!live || (unsigned)y >= (unsigned)g.ny || (unsigned)z >= (unsigned)g.nz) continue;
+            unsigned long long* row = acc + ((int64_t)z * g.ny + y) * g.nx;
+            if ((unsigned)c.i0 < (unsigned)g.nx) red_add(row + c.i0, lo);
+            if (!give && (unsigned)(c.i0 + 1) < (unsigned)g.nx) red_add(row + c.i0 + 1, hi);
+        }
+    }
+}
+
+// Adjoint of mbc_combine for up to PG views from p0 on, L <= 4 levels: one pass
+// reads E and the views' d_dvf and forms both gradients -- d_mbc per voxel
+// (continued from its stored sum when p0 > 0, so the views add in order) and
+// the 3 L PG coefficient sums per thread, reduced over the block in a fixed
+// order into part[output][block].  Bandwidth bound; the two passes it replaces
+// read d_dvf twice and E per view and took 76 + 68 us at the paper grid (one
+// fp32 view), and a single thread per output summed the 608 partials in 53 us:
+// 54 us now, 336 MB being 50 us at the copy rate.  PG = 1 takes four voxels
+// per thread, PG = 4 two, what their sums leave registers for.
+template <typename T, int L, int PG, int V>
+__global__ void __launch_bounds__(kThreads, 2) k_combine_bwd(GridD g, int P, int p0, const T* __restrict__ E,
+                                                          const float* __restrict__ w, const float* __restrict__ dD,
+                                                          float* dE, float* part, int accumulate) {
+    constexpr int K = 3 * L;
+    __shared__ float red[kThreads / 32][PG * K];
+    const int64_t N = g.n;
+    const int np = min(PG, P - p0);
+    float acc[PG][K];
+#pragma unroll
+    for (int q = 0; q < PG; q++)
+#pragma unroll
+        for (int c = 0; c < K; c++) acc[q][c] = 0.f;
+    for (int64_t v = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); v < N;
+         v += V * (int64_t)gridDim.x * blockDim.x) {
+        float dd[PG][3][V];
+#pragma unroll
+        for (int q = 0; q < PG; q++)
+            if (q < np) {
+#pragma unroll
+                for (int k = 0; k < 3; k++) ld_run<V>(dD + ((int64_t)(p0 + q) * 3 + k) * N + v, dd[q][k]);
+            }
+#pragma unroll
+        for (int c = 0; c < K; c++) {  // c = 3 l + k
+            float e[V], gE[V];
+            ld_run<V>(E + (int64_t)c * N + v, e);
+#pragma unroll
+            for (int i = 0; i < V; i++) gE[i] = 0.f;
+            float* o = dE + (int64_t)c * N + v;
+            const bool more = accumulate || p0 > 0;
+            float old[V];
+            if (more) {
+#pragma unroll
+                for (int i = 0; i < V; i++) old[i] = o[i];
+                if (p0 > 0) {
+#pragma unroll
+                    for (int i = 0; i < V; i++) gE[i] = old[i];
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < PG; q++)
+                if (q < np) {
+                    const float cw = __ldg(w + (int64_t)(p0 + q) * K + c);
+#pragma unroll
+                    for (int i = 0; i < V; i++) {
+                        gE[i] = fmaf(dd[q][c % 3][i], cw, gE[i]);
+                        acc[q][c] = fmaf(dd[q][c % 3][i], e[i], acc[q][c]);
+                    }
+                }
+            if (more && p0 == 0) {
+#pragma unroll
+                for (int i = 0; i < V; i++) gE[i] = old[i] + gE[i];
+            }
+            st_run<V>(o, gE);
+        }
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, slot = split_slot<K>(lane);
+#pragma unroll
+    for (int q = 0; q < PG; q++) {
+        SplitReduce<K, 16>::run(acc[q], lane);
+        if (slot >= 0) red[warp][q * K + slot] = acc[q][0];
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < np * K; c += kThreads) {
+        float r = 0.f;
+        for (int wi = 0; wi < kThreads / 32; wi++) r += red[wi][c];
+        part[((int64_t)p0 * K + c) * gridDim.x + blockIdx.x] = r;
+    }
+}
+
 // One CTA per output: strided fixed-order partial sums, then a fixed tree,
 // in double (the tile partials of a coefficient gradient cancel heavily).
 __global__ void __launch_bounds__(256) k_reduce_partials_wide(const float* part, int nb, float* out, int accumulate) {
@@ -843,6 +1073,68 @@ __global__ void __launch_bounds__(256) k_reduce_partials_wide(const float* part,
     }
 }
 
+unsigned stream_blocks(int64_t work) {
+    int64_t b = (work + kThreads - 1) / kThreads;
+    return (unsigned)(b < kStreamBlocks ? (b > 0 ? b : 1) : kStreamBlocks);
+}
+
+template <typename T>
+void launch_combine(const GridD& g, int L, int P, const void* mbc, const float* coeff, void* dvf, cudaStream_t s) {
+    const T* E = (const T*)mbc;
+    T* D = (T*)dvf;
+    const bool run4 = runs_aligned<4>(g.n, mbc, dvf);
+    const unsigned nb = stream_blocks(run4 ? (g.n + 3) / 4 : g.n);
+#define PMF_COMBINE(LL)                                                                       \
+    if (run4) k_combine<T, LL, 4><<<nb, kThreads, 0, s>>>(g, L, P, E, coeff, D);              \
+    else k_combine<T, LL, 1><<<nb, kThreads, 0, s>>>(g, L, P, E, coeff, D);                   \
+    break;
+    switch (L) {
+        case 1: PMF_COMBINE(1)
+        case 2: PMF_COMBINE(2)
+        case 3: PMF_COMBINE(3)
+        case 4: PMF_COMBINE(4)
+        default: k_combine<T, 0, 1><<<stream_blocks(g.n), kThreads, 0, s>>>(g, L, P, E, coeff, D);
+    }
+#undef PMF_COMBINE
+}
+
+template <typename T, int L>
+void launch_combine_bwd_level(const GridD& g, int P, const T* E, const float* coeff, const float* d_dvf, float* d_mbc,
+                              float* part, int accumulate, cudaStream_t s) {
+    // every block writes its partial of every output, so kStreamBlocks partials
+    // are always summed whatever the grid
+    for (int p0 = 0; p0 < P; p0 += P == 1 ? 1 : 4) {
+        const bool run = runs_aligned<4>(g.n, E, d_dvf) && (((uintptr_t)d_mbc) & 15) == 0;
+        if (P == 1 && run)
+            k_combine_bwd<T, L, 1, 4><<<kStreamBlocks, kThreads, 0, s>>>(g, P, p0, E, coeff, d_dvf, d_mbc, part, accumulate);
+        else if (P == 1)
+            k_combine_bwd<T, L, 1, 1><<<kStreamBlocks, kThreads, 0, s>>>(g, P, p0, E, coeff, d_dvf, d_mbc, part, accumulate);
+        else if (run)
+            k_combine_bwd<T, L, 4, 2><<<kStreamBlocks, kThreads, 0, s>>>(g, P, p0, E, coeff, d_dvf, d_mbc, part, accumulate);
+        else
+            k_combine_bwd<T, L, 4, 1><<<kStreamBlocks, kThreads, 0, s>>>(g, P, p0, E, coeff, d_dvf, d_mbc, part, accumulate);
+    }
+}
+
+// Both gradients of mbc_combine; part: [P L 3][kStreamBlocks] floats.  More than
+// four levels (whose sums would not fit the one-pass kernel's registers) take
+// the two-pass kernels.
+template <typename T>
+void launch_combine_bwd(const GridD& g, int L, int P, const void* mbc, const float* coeff, const float* d_dvf,
+                        float* d_mbc, float* d_coeff, float* part, int accumulate, cudaStream_t s) {
+    const T* E = (const T*)mbc;
+    switch (L) {
+        case 1: launch_combine_bwd_level<T, 1>(g, P, E, coeff, d_dvf, d_mbc, part, accumulate, s); break;
+        case 2: launch_combine_bwd_level<T, 2>(g, P, E, coeff, d_dvf, d_mbc, part, accumulate, s); break;
+        case 3: launch_combine_bwd_level<T, 3>(g, P, E, coeff, d_dvf, d_mbc, part, accumulate, s); break;
+        case 4: launch_combine_bwd_level<T, 4>(g, P, E, coeff, d_dvf, d_mbc, part, accumulate, s); break;
+        default:
+            k_combine_bwd_mbc<<<stream_blocks(g.n), kThreads, 0, s>>>(g, L, P, coeff, d_dvf, d_mbc, accumulate);
+            k_combine_bwd_coeff<T><<<dim3(kStreamBlocks, (unsigned)(P * 3)), kThreads, 0, s>>>(g, L, P, E, d_dvf, part);
+    }
+    k_reduce_partials_wide<<<(unsigned)(P * L * 3), 256, 0, s>>>(part, kStreamBlocks, d_coeff, accumulate);
+}
+
 template <typename T, int LL>
 void launch_wc_bwd(unsigned nt, size_t smem, cudaStream_t s, const GridD& g, int P, const void* ref, const void* mbc,
                    const float* coeff, const float* d_out, float* d_mbc, unsigned long long* acc,
@@ -850,11 +1142,6 @@ void launch_wc_bwd(unsigned nt, size_t smem, cudaStream_t s, const GridD& g, int
     cudaFuncSetAttribute(k_wc_bwd_tile<T, LL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_wc_bwd_tile<T, LL><<<nt, GeomBwd::THREADS, smem, s>>>(g, P, (const T*)ref, (const T*)mbc, coeff, d_out, d_mbc, acc, maxbits,
                                                 part, accumulate);
-}
-
-unsigned stream_blocks(int64_t work) {
-    int64_t b = (work + kThreads - 1) / kThreads;
-    return (unsigned)(b < kStreamBlocks ? (b > 0 ? b : 1) : kStreamBlocks);
 }
 
 pmf_status check_common(const pmf_grid* grid, int32_t P, pmf_dtype dtype) {
@@ -884,7 +1171,7 @@ pmf_status mbc_combine(const pmf_grid* grid, int32_t L, int32_t P, pmf_dtype dty
     PMF_REQUIRE(mbc && coeff && dvf, "null pointer");
     GridD g = make_grid(grid);
     cudaStream_t s = (cudaStream_t)stream;
-    PMF_DISPATCH_DTYPE(dtype, T, k_combine<T><<<stream_blocks(g.n), kThreads, 0, s>>>(g, L, P, (const T*)mbc, coeff, (T*)dvf));
+    PMF_DISPATCH_DTYPE(dtype, T, launch_combine<T>(g, L, P, mbc, coeff, dvf, s));
     return check_launch("mbc_combine");
 }
 
@@ -913,12 +1200,7 @@ pmf_status mbc_combine_backward(const pmf_grid* grid, int32_t L, int32_t P, pmf_
         if (!accumulate) cudaMemsetAsync(d_mbc, 0, sizeof(float) * (size_t)(L * 3 * g.n), s);
         return check_launch("mbc_combine_backward");
     }
-    k_combine_bwd_mbc<<<stream_blocks(g.n), kThreads, 0, s>>>(g, L, P, coeff, d_dvf, d_mbc, accumulate);
-    dim3 gr(kStreamBlocks, (unsigned)(P * 3));
-    float* part = (float*)ws;
-    PMF_DISPATCH_DTYPE(dtype, T, k_combine_bwd_coeff<T><<<gr, kThreads, 0, s>>>(g, L, P, (const T*)mbc, d_dvf, part));
-    int64_t nout = (int64_t)P * L * 3;
-    k_reduce_partials<<<(unsigned)((nout + 255) / 256), 256, 0, s>>>(part, nout, kStreamBlocks, d_coeff, accumulate);
+    PMF_DISPATCH_DTYPE(dtype, T, launch_combine_bwd<T>(g, L, P, mbc, coeff, d_dvf, d_mbc, d_coeff, (float*)ws, accumulate, s));
     return check_launch("mbc_combine_backward");
 }
 
@@ -930,7 +1212,12 @@ pmf_status warp_volume(const pmf_grid* grid, int32_t P, pmf_dtype dtype, const v
     PMF_REQUIRE(ref && dvf && out, "null pointer");
     GridD g = make_grid(grid);
     cudaStream_t s = (cudaStream_t)stream;
-    PMF_DISPATCH_DTYPE(dtype, T, k_warp<T><<<stream_blocks(g.n * P), kThreads, 0, s>>>(g, P, (const T*)ref, (const T*)dvf, (T*)out));
+    const WarpTiles nt = warp_tiles(g);
+    const int per = views_per_launch(nt);
+    for (int p0 = 0; p0 < P; p0 += per) {
+        const int np = P - p0 < per ? P - p0 : per;
+        PMF_DISPATCH_DTYPE(dtype, T, k_warp<T><<<nt.per_view() * (unsigned)np, kThreads, 0, s>>>(g, nt, (const T*)ref, (const T*)dvf + (int64_t)p0 * 3 * g.n, (T*)out + (int64_t)p0 * g.n));
+    }
     return check_launch("warp_volume");
 }
 
@@ -959,7 +1246,12 @@ pmf_status warp_volume_backward(const pmf_grid* grid, int32_t P, pmf_dtype dtype
     cudaMemsetAsync(ws, 0, need, s);
     if (P > 0) {
         k_absmax<<<stream_blocks(g.n * P), kThreads, 0, s>>>(d_out, g.n * P, maxbits);
-        PMF_DISPATCH_DTYPE(dtype, T, k_warp_bwd<T><<<stream_blocks(g.n * P), kThreads, 0, s>>>(g, P, (const T*)ref, (const T*)dvf, d_out, d_dvf, acc, maxbits, accumulate));
+        const WarpTiles nt = warp_tiles(g);
+        const int per = views_per_launch(nt);
+        for (int p0 = 0; p0 < P; p0 += per) {
+            const int np = P - p0 < per ? P - p0 : per;
+            PMF_DISPATCH_DTYPE(dtype, T, k_warp_bwd<T><<<nt.per_view() * (unsigned)np, kThreads, 0, s>>>(g, nt, (const T*)ref, (const T*)dvf + (int64_t)p0 * 3 * g.n, d_out + (int64_t)p0 * g.n, d_dvf ? d_dvf + (int64_t)p0 * 3 * g.n : nullptr, acc, maxbits, (float)(g.n * (int64_t)P), accumulate));
+        }
     }
     k_fixed_to_float<<<stream_blocks(g.n), kThreads, 0, s>>>(acc, g.n, maxbits, (float)(g.n * (int64_t)P), d_ref, accumulate);
     return check_launch("warp_volume_backward");
@@ -1211,12 +1503,8 @@ extern "C" pmf_status mbc_combine_backward_noalloc(const pmf_grid* grid, int32_t
     }
     float* part = nullptr;
     if ((st = noalloc_scratch(&part)) != PMF_OK) return st;
-    // every partial slot the reduction reads is written by k_combine_bwd_coeff
-    // first, so the array needs no clearing between calls
-    k_combine_bwd_mbc<<<stream_blocks(g.n), kThreads, 0, s>>>(g, L, P, coeff, d_dvf, d_mbc, accumulate);
-    dim3 gr(kStreamBlocks, (unsigned)(P * 3));
-    PMF_DISPATCH_DTYPE(dtype, T, k_combine_bwd_coeff<T><<<gr, kThreads, 0, s>>>(g, L, P, (const T*)mbc, d_dvf, part));
-    const int64_t nout = (int64_t)P * L * 3;
-    k_reduce_partials<<<(unsigned)((nout + 255) / 256), 256, 0, s>>>(part, nout, kStreamBlocks, d_coeff, accumulate);
+    // every partial slot the reduction reads is written by the pass before it,
+    // so the array needs no clearing between calls
+    PMF_DISPATCH_DTYPE(dtype, T, launch_combine_bwd<T>(g, L, P, mbc, coeff, d_dvf, d_mbc, d_coeff, part, accumulate, s));
     return check_launch("mbc_combine_backward_noalloc");
 }

@@ -579,3 +579,41 @@ def test_voxelize_backward_unsplit_many_gaussians():
     ref = oracle.voxelize_backward(grid, gs.mean, gs.scale, gs.quat, gs.value, d_out, 3.0)
     for name, g_, r_ in zip(("mean", "scale", "quat", "value"), got, ref):
         assert rel_l2(host(g_), r_) <= 1e-4, name
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("n,L,P", [((8, 4, 3), 1, 1), ((8, 4, 3), 3, 2), ((7, 5, 3), 2, 1), ((7, 5, 3), 4, 5),
+                                   ((33, 9, 5), 3, 4), ((12, 5, 4), 5, 3), ((12, 5, 4), 4, 9)])
+def test_unfused_calls_at_run_and_tile_edges(n, L, P, dt):
+    """mbc_combine, warp_volume and their adjoints where the four-voxel runs end
+    (N a multiple of four or odd), past the 32 x 8 x 2 warp tile and the 8 x 16 x 4
+    adjoint tile, for one view, a full group of four, a group and a rest, and
+    more than four levels; displacements of up to a few voxels, some beyond the
+    adjoint's 4-voxel halo.  fp32 sums: 1e-5 relative (reduced inputs are
+    compared from the stored values, a reduced DVF to its half-ulp)."""
+    grid = Grid(*n, 2.0, 2.0, 2.0)
+    V, E, w = _mbc_and_ref(grid, 300 + L, L=L, P=P)
+    Vd, Ed = dev(V).to(dt), dev(3.0 * E).to(dt)
+    Vq, Eq = host(Vd), host(Ed)
+    eps = {torch.float32: 1e-6, torch.bfloat16: 2.0 ** -8, torch.float16: 2.0 ** -11}[dt]
+    D = pmf.mbc_combine(grid, Ed, dev(w))
+    assert rel_l2(host(D), oracle.combine(Eq, w)) <= eps
+    Dq = host(D)
+    W = pmf.warp_volume(grid, Vd, D)
+    assert rel_l2(host(W), oracle.warp(grid, Vq, Dq)) <= (TOL32 if dt == torch.float32 else eps)
+    rng = np.random.default_rng(310 + P)
+    dW = rng.normal(size=(P,) + grid.shape).astype(np.float32)
+    dV, dD = pmf.warp_volume_backward(grid, Vd, D, dev(dW))
+    dV_ref, dD_ref = oracle.warp_backward(grid, Vq, Dq, dW)
+    assert rel_l2(host(dV), dV_ref) <= TOL32
+    assert rel_l2(host(dD), dD_ref) <= 1e-4
+    dV2, none = pmf.warp_volume_backward(grid, Vd, D, dev(dW), need_dvf=False)
+    assert none is None and torch.equal(dV, dV2)
+    g = rng.normal(size=(P, 3) + grid.shape).astype(np.float32)
+    dE, dw = pmf.mbc_combine_backward(grid, Ed, dev(w), dev(g))
+    dE_ref, dw_ref = oracle.combine_backward(Eq, w, g)
+    assert rel_l2(host(dE), dE_ref) <= 1e-6
+    assert rel_l2(host(dw), dw_ref) <= 1e-5
+    base = (dE.clone(), dw.clone())
+    pmf.mbc_combine_backward(grid, Ed, dev(w), dev(g), accumulate=True, grads=base)
+    assert rel_l2(host(base[0]), 2.0 * dE_ref) <= 1e-6 and rel_l2(host(base[1]), 2.0 * dw_ref) <= 1e-5
