@@ -202,18 +202,19 @@ __device__ __forceinline__ int plane_stride(int rows, int pitch) {
 // The samples j0..j1 of one ray of the chunk into a box with rows PITCH words
 // apart (a template argument, so the corner offsets are immediates) and NBOX
 // words in all.
-template <int PITCH, int NBOX>
-__device__ __forceinline__ void scatter_samples(const Ray& r, const Box& bx, int sz, bool mirror, float sxf, float gsb,
-                                                int j0, int j1, const int ib[3], const float fb[3], int* box) {
-    constexpr int sy = PITCH;
-    const float syf = (float)sy, szf = (float)sz;
+template <int PITCH, bool MIRROR, int NBOX>
+__device__ __forceinline__ void scatter_samples(const Ray& r, const Box& bx, int sz, float gsb, int j0, int j1,
+                                                const int ib[3], const float fb[3], int* box) {
     // positions relative to the anchor cell, bounded like the box.
     // Box column of voxel x: x - lx, or bx - 1 - (x - lx) mirrored;
     // a sample's base address is its cell's lower-x corner, or its
     // upper-x corner when mirrored, so the corners always sit at
-    // +0, +1, +sy, +sy + 1 (the two x weights trade places)
-    int* qa = box + (mirror ? bx.bx - 2 - (ib[0] - bx.lx) : ib[0] - bx.lx) + (ib[1] - bx.ly) * sy +
-              (ib[2] - bx.lz) * sz;
+    // +0, +1, +sy, +sy + 1 (the two x weights trade places).
+    // The cell comes from the positions' floor bits (kFloorBias), whose biases
+    // off takes out again modulo 2^32.
+    const int col = MIRROR ? bx.bx - 2 - (ib[0] - bx.lx) : ib[0] - bx.lx;
+    const unsigned off = (unsigned)(col + (ib[1] - bx.ly) * PITCH + (ib[2] - bx.lz) * sz) -
+                         kFloorBits * ((MIRROR ? 0u - 1u : 1u) + (unsigned)PITCH + (unsigned)sz);
     // every sample adds its 8 scaled corner weights to the box; the
     // weights are formed with the bias kMagic, so each rounds to an
     // integer-valued float and converts with one integer subtract.
@@ -224,20 +225,26 @@ __device__ __forceinline__ void scatter_samples(const Ray& r, const Box& bx, int
     // stagger (taken modulo its count) and wrapping, so a chunk the
     // ray only enters or leaves costs no idle iterations
     const int len = j1 - j0 + 1;
-    int jj = adjoint_phase() % len;
+    const float jfirst = (float)j0, jlast = (float)j1;
+    float jf = (float)(j0 + adjoint_phase() % len);
+    const f32x2 dxy = pack2(r.dh[0], r.dh[1]), bxy = pack2(fb[0], fb[1]), M2 = pack2(kFloorBias, kFloorBias);
+    const f32x2 one2 = pack2(1.0f, 1.0f);
+#pragma unroll 2  // two samples' chains interleave
     for (int k = 0; k < len; k++) {
-        const int j = j0 + jj;
-        jj = jj + 1 == len ? 0 : jj + 1;
-        const float jf = (float)j;
-        const float ux = fmaf(jf, r.dh[0], fb[0]), uy = fmaf(jf, r.dh[1], fb[1]),
-                    uz = fmaf(jf, r.dh[2], fb[2]);
-        const float flx = floorf(ux), fly = floorf(uy), flz = floorf(uz);
-        const int idx = (int)fmaf(flx, sxf, fmaf(fly, syf, flz * szf));
-        const float fx = ux - flx, fy = uy - fly, fz = uz - flz;
-        const float ex = 1.0f - fx, ey = 1.0f - fy, ez = (1.0f - fz) * gsb, fzs = fz * gsb;
+        const f32x2 uxy = fma2(pack2(jf, jf), dxy, bxy);
+        const float uz = fmaf(jf, r.dh[2], fb[2]);
+        jf = jf == jlast ? jfirst : jf + 1.0f;
+        const f32x2 txy = add2_down(uxy, M2);
+        const float tz = __fadd_rd(uz, kFloorBias);
+        const unsigned bx_ = __float_as_uint(lo2(txy));
+        const int idx = (int)(__float_as_uint(tz) * (unsigned)sz +
+                              (__float_as_uint(hi2(txy)) * (unsigned)PITCH + (MIRROR ? off - bx_ : off + bx_)));
+        const f32x2 fxy = sub2(uxy, sub2(txy, M2)), exy = sub2(one2, fxy);
+        const float fx = lo2(fxy), fy = hi2(fxy), ex = lo2(exy), ey = hi2(exy), fz = uz - (tz - kFloorBias);
+        const float ez = (1.0f - fz) * gsb, fzs = fz * gsb;
         const float a0 = ey * ez, a1 = fy * ez, a2 = ey * fzs, a3 = fy * fzs;
-        const float w0 = mirror ? fx : ex, w1 = mirror ? ex : fx;  // the corners at +0 and +1
-        int* q = qa + idx;
+        const float w0 = MIRROR ? fx : ex, w1 = MIRROR ? ex : fx;  // the corners at +0 and +1
+        int* q = box + idx;
         int* q2 = q + sz;
         if (!PMF_DCHECK(q >= box && q2 + PITCH + 1 < box + NBOX)) continue;
         atomicAdd(q, __float_as_int(fmaf(w0, a0, kMagic)) - kMagicBits);
@@ -304,7 +311,6 @@ __device__ __forceinline__ void backproject_tile(const GridD& g, int nu, int nv,
     const int Mlo = bs.range[0], Mhi = bs.range[1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool mirror = tile_mirror<RPB>(views[p], nu, nv, ntu, tile);
-    const float sxf = mirror ? -1.0f : 1.0f;
     int sel = 0;
     for (int M0 = Mlo; M0 <= Mhi; M0 += CH, sel ^= 1) {
         int j0, j1, ib[3];
@@ -318,8 +324,10 @@ __device__ __forceinline__ void backproject_tile(const GridD& g, int nu, int nv,
         if (threadIdx.x == 0 && bx.vol > 0 && !fits) diag_count(PMF_DIAG_BACKPROJECT_BOX_FALLBACK);
         if (fits) {
             if (act) {
-                if (pitch == 33) scatter_samples<33, box_words<CH>()>(r, bx, sz, mirror, sxf, gsb, j0, j1, ib, fb, box);
-                else scatter_samples<65, box_words<CH>()>(r, bx, sz, mirror, sxf, gsb, j0, j1, ib, fb, box);
+                if (pitch == 33 && mirror) scatter_samples<33, true, box_words<CH>()>(r, bx, sz, gsb, j0, j1, ib, fb, box);
+                else if (pitch == 33) scatter_samples<33, false, box_words<CH>()>(r, bx, sz, gsb, j0, j1, ib, fb, box);
+                else if (mirror) scatter_samples<65, true, box_words<CH>()>(r, bx, sz, gsb, j0, j1, ib, fb, box);
+                else scatter_samples<65, false, box_words<CH>()>(r, bx, sz, gsb, j0, j1, ib, fb, box);
             }
             __syncthreads();
             // flush the box: lane = x, one warp per (y, z) row; one 64-bit atomic
