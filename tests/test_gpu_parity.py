@@ -617,3 +617,18 @@ def test_unfused_calls_at_run_and_tile_edges(n, L, P, dt):
     base = (dE.clone(), dw.clone())
     pmf.mbc_combine_backward(grid, Ed, dev(w), dev(g), accumulate=True, grads=base)
     assert rel_l2(host(base[0]), 2.0 * dE_ref) <= 1e-6 and rel_l2(host(base[1]), 2.0 * dw_ref) <= 1e-5
+
+
+@pytest.mark.parametrize("C", [1, 3])
+@pytest.mark.parametrize("n,G,scale", [((37, 5, 3), 7, (0.4, 1.5)), ((150, 40, 30), 3, (8.0, 30.0))])
+def test_voxelize_backward_row_plans(n, G, scale, C):
+    """The adjoint numbers the blocks of 64 box rows at a time and lists 512 of
+    them: a few rows, and rows as long as the grid (several listings per plan);
+    against the oracle within the gradient bounds used above."""
+    grid = Grid(*n, 2.0, 2.0, 2.0)
+    gs = _rand_gaussians(400 + G, grid, G, scale[0] * 2.0, scale[1] * 2.0, C)
+    d = np.random.default_rng(401 + G).normal(size=(C,) + grid.shape).astype(np.float32)
+    got = pmf.gs_voxelize_backward(grid, gset(gs, 3.0), dev(d))
+    ref = oracle.voxelize_backward(grid, gs.mean, gs.scale, gs.quat, gs.value, d, 3.0)
+    for x, r in zip(got, ref):
+        assert rel_l2(host(x), np.asarray(r).reshape(tuple(x.shape))) <= 1e-4
