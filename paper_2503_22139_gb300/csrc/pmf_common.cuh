@@ -307,11 +307,20 @@ __device__ __forceinline__ void red_add(unsigned long long* p, unsigned long lon
 __device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
 
 // Grid-stride maximum of |x[0..n)| into *out as abs_bits (every thread of the
-// launch calls it; blocks are whole warps).
+// launch calls it; blocks are whole warps): 16-byte loads between the first and
+// last 16-byte boundary, four in flight per thread, the ends one by one.
 __device__ __forceinline__ void absmax_bits(const float* __restrict__ x, int64_t n, unsigned* out) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    const int64_t lead = (4 - (int64_t)(((uintptr_t)x >> 2) & 3)) & 3, head = lead < n ? lead : n;
+    const int64_t n4 = (n - head) >> 2, tail = head + 4 * n4;
+    const float4* x4 = reinterpret_cast<const float4*>(x + head);
     unsigned m = 0u;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, abs_bits(__ldg(x + t)));
+#pragma unroll 4
+    for (int64_t t = t0; t < n4; t += nt) {
+        const float4 v = __ldg(x4 + t);
+        m = max(max(max(m, abs_bits(v.x)), max(abs_bits(v.y), abs_bits(v.z))), abs_bits(v.w));
+    }
+    for (int64_t t = t0; t < head + (n - tail); t += nt) m = max(m, abs_bits(__ldg(x + (t < head ? t : tail + (t - head)))));
     m = __reduce_max_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
 }
