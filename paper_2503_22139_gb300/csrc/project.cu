@@ -14,34 +14,99 @@ namespace {
 // ----------------------------------------------------------------- forward
 
 // Capacity (floats) of the plain-staging box, in dynamic shared memory: a
-// 48-sample chunk's box at the paper geometry, with rows of 33 floats (65 when
-// the box is wider than 32 voxels, the same bank pattern).
+// 48-sample chunk's box at the paper geometry.
 constexpr int kPlainBox = 13312;
+
+// Row pitch of the bulk-copied box, and of the plain-staged one where it fits:
+// rows 12 banks and planes 16 banks apart put the 4 x 4 x 2 voxels around any
+// point in 32 distinct banks.
+constexpr int kTmaX = 44;
 
 // The staged samples [j0, j1] of one ray on a box with rows PITCH floats apart
 // and planes sz floats apart (PITCH a template argument, so the corner offsets
-// are immediates).
-template <int PITCH>
-__device__ __forceinline__ void gather_samples(const Ray& r, const float* box, const Box& bx, int sz, int j0, int j1,
-                                               const int ib[3], const float fb[3], float& acc) {
-    // positions relative to the anchor cell; the box was bounded with the same
-    // expression, so every cell is inside it
+// are immediates); q0 is the anchor cell's corner.  Positions are relative to
+// the anchor cell; the box was bounded with the same expression, so every cell
+// is inside it.  The x/y position and the z-paired blends are packed fp32 pairs
+// ((a00, a01), (a10, a11), then (b0, b1)): the scalar operations' bits in fewer
+// instructions.  BULK (the bulk-copied box) takes x's floor and the cell index
+// from the bits of biased floats (kFloorBias), which moves half of the
+// conversion pipe's work (57% busy) to the fp32 pipe, and interleaves three
+// samples: 3,730 -> 3,624 us for 32 fp32 views at the paper geometry (all floors
+// that way: 3,880).  The plain-staged kernel, with more live registers, is 2-4%
+// slower so and keeps the conversions and two samples.  Same values either way.
+template <int PITCH, int NBOX, bool BULK>
+__device__ __forceinline__ void gather_samples(const Ray& r, const float* box, const float* q0, int sz, int j0, int j1,
+                                               const float fb[3], float& acc) {
     constexpr int sy = PITCH;
     const float syf = (float)sy, szf = (float)sz;
-    const float* qa = box + (ib[0] - bx.lx) + (ib[1] - bx.ly) * sy + (ib[2] - bx.lz) * sz;
-    float jf = (float)j0;
-    for (int j = j0; j <= j1; j++, jf += 1.0f) {
-        const float ux = fmaf(jf, r.dh[0], fb[0]), uy = fmaf(jf, r.dh[1], fb[1]), uz = fmaf(jf, r.dh[2], fb[2]);
-        const float flx = floorf(ux), fly = floorf(uy), flz = floorf(uz);
-        const float fx = ux - flx, fy = uy - fly, fz = uz - flz;
-        const float* q = qa + (int)fmaf(flz, szf, fmaf(fly, syf, flx));
-        if (!PMF_DCHECK(q >= box && q + sz + sy + 1 < box + kPlainBox)) continue;
-        const float c000 = q[0], c100 = q[1], c010 = q[sy], c110 = q[sy + 1];
-        const float c001 = q[sz], c101 = q[sz + 1], c011 = q[sz + sy], c111 = q[sz + sy + 1];
-        const float a00 = fmaf(fx, c100 - c000, c000), a10 = fmaf(fx, c110 - c010, c010);
-        const float a01 = fmaf(fx, c101 - c001, c001), a11 = fmaf(fx, c111 - c011, c011);
-        const float b0 = fmaf(fy, a10 - a00, a00), b1 = fmaf(fy, a11 - a01, a01);
+    const f32x2 dxy = pack2(r.dh[0], r.dh[1]), bxy = pack2(fb[0], fb[1]), one = pack2(1.0f, 1.0f);
+    f32x2 jj = pack2((float)j0, (float)j0);
+#pragma unroll (BULK ? 3 : 2)
+    for (int j = j0; j <= j1; j++, jj = add2(jj, one)) {
+        const f32x2 uxy = fma2(jj, dxy, bxy);
+        const float ux = lo2(uxy), uy = hi2(uxy), uz = fmaf(lo2(jj), r.dh[2], fb[2]);
+        const float tx = BULK ? __fadd_rd(ux, kFloorBias) : 0.0f;
+        const float flx = BULK ? tx - kFloorBias : floorf(ux), fly = floorf(uy), flz = floorf(uz);
+        const f32x2 fxy = sub2(uxy, pack2(flx, fly));
+        const float fx = lo2(fxy), fy = hi2(fxy), fz = uz - flz;
+        const float at = fmaf(flz, szf, fmaf(fly, syf, BULK ? tx : flx));  // exact: integers below 2^22
+        const float* q = q0 + (BULK ? __float_as_int(at) - (int)kFloorBits : (int)at);
+        if (!PMF_DCHECK(q >= box && q + sz + sy + 1 < box + NBOX)) continue;
+        const f32x2 c00 = pack2(q[0], q[sz]), c10 = pack2(q[1], q[sz + 1]);
+        const f32x2 c01 = pack2(q[sy], q[sz + sy]), c11 = pack2(q[sy + 1], q[sz + sy + 1]);
+        const f32x2 fx2 = pack2(fx, fx);
+        const f32x2 a0 = fma2(fx2, sub2(c10, c00), c00), a1 = fma2(fx2, sub2(c11, c01), c01);
+        const f32x2 bb = fma2(pack2(fy, fy), sub2(a1, a0), a0);
+        const float b0 = lo2(bb), b1 = hi2(bb);
         acc += fmaf(fz, b1 - b0, b0);  // into the tile's sum in sample order, as every path does
+    }
+}
+
+// Layout of a plain-staged box: the bulk copies' pitch and plane skew where the
+// box fits with them, else rows of 33 or, for boxes wider than 32 voxels, 65
+// floats (one bank per row); 0 if none fits.  (The plain form had only the
+// latter, with 1.3 wavefronts per load, and a scalar blend: four fp32 volumes of
+// odd sizes, 16 views, both ways: 3,565 -> 3,390 us.)
+__device__ __forceinline__ int plain_layout(const Box& bx, int& sz) {
+    sz = bx.by * kTmaX;
+    sz += (16 - sz) & 31;
+    if (bx.bx <= kTmaX && (long long)bx.bz * sz <= kPlainBox) return kTmaX;
+    const int pitch = bx.bx <= 32 ? 33 : 65;
+    sz = pitch * bx.by;
+    return bx.bx <= 64 && (long long)bx.bz * sz <= kPlainBox ? pitch : 0;
+}
+
+// Stages the box with plain loads: lane = x (two passes when wider than 32), one
+// warp per (y, z) row, four rows' loads in flight, zero outside the grid.
+template <typename T, int RPB>
+__device__ __forceinline__ void stage_plain(const T* __restrict__ V, const GridD& g, const Box& bx, int pitch, int sz,
+                                            float* box) {
+    constexpr int W = RPB / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rows = bx.by * bx.bz;
+    for (int col = lane; col < bx.bx; col += 32) {
+        const int x = bx.lx + col;
+        const bool xin = (unsigned)x < (unsigned)g.nx;
+        int zz = warp / bx.by, yy = warp - zz * bx.by;
+        for (int row = warp; row < rows; row += 4 * W) {
+            float v[4];
+            int at[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int y = bx.ly + yy, z = bx.lz + zz;
+                const bool valid = row + u * W < rows;
+                at[u] = valid ? zz * sz + yy * pitch + col : -1;
+                v[u] = valid && xin && (unsigned)y < (unsigned)g.ny && (unsigned)z < (unsigned)g.nz
+                           ? Store<T>::ld(V, (z * g.ny + y) * g.nx + x) : 0.0f;  // N < 2^31
+                yy += W;
+                while (yy >= bx.by) {
+                    yy -= bx.by;
+                    zz++;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (at[u] >= 0 && PMF_DCHECK(at[u] < kPlainBox)) box[at[u]] = v[u];
+        }
     }
 }
 
@@ -65,7 +130,6 @@ __device__ __forceinline__ void project_tile(const GridD& g, int nu, int nv, int
     const T* V = vol + (int64_t)p * vol_stride;
     block_range(bs, r, live);
     const int Mlo = bs.range[0], Mhi = bs.range[1];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float acc = 0.0f;
     int sel = 0;
     for (int M0 = Mlo; M0 <= Mhi; M0 += CH, sel ^= 1) {
@@ -74,33 +138,18 @@ __device__ __forceinline__ void project_tile(const GridD& g, int nu, int nv, int
         const bool act = chunk_begin<CH>(bs, sel, r, live, M0, j0, j1, ib, fb);
         __syncthreads();
         const Box bx = read_box(bs, sel);
-        const int pitch = bx.bx <= 32 ? 33 : 65;
-        const int sz = pitch * bx.by;
-        const bool fits = bx.vol > 0 && bx.bx <= 64 && (long long)bx.bz * sz <= kPlainBox;
+        int sz;
+        const int pitch = bx.vol > 0 ? plain_layout(bx, sz) : 0;
+        const bool fits = pitch > 0;
         if (threadIdx.x == 0 && bx.vol > 0 && !fits) diag_count(PMF_DIAG_PROJECT_BOX_FALLBACK);
         if (fits) {
-            // stage the box: lane = x (two passes when wider than 32), one warp
-            // per (y, z) row, zero outside the grid
-            for (int col = lane; col < bx.bx; col += 32) {
-                const int x = bx.lx + col;
-                const bool xin = (unsigned)x < (unsigned)g.nx;
-                for (int zz = 0; zz < bx.bz; zz++) {
-                    const int z = bx.lz + zz;
-                    const bool zin = (unsigned)z < (unsigned)g.nz;
-                    for (int yy = warp; yy < bx.by; yy += RPB / 32) {
-                        const int y = bx.ly + yy;
-                        float val = 0.0f;
-                        if (xin && zin && (unsigned)y < (unsigned)g.ny)
-                            val = Store<T>::ld(V, ((int64_t)z * g.ny + y) * g.nx + x);
-                        const int i = zz * sz + yy * pitch + col;
-                        if (PMF_DCHECK(i < kPlainBox)) box[i] = val;
-                    }
-                }
-            }
+            stage_plain<T, RPB>(V, g, bx, pitch, sz, box);
             __syncthreads();
             if (act) {
-                if (pitch == 33) gather_samples<33>(r, box, bx, sz, j0, j1, ib, fb, acc);
-                else gather_samples<65>(r, box, bx, sz, j0, j1, ib, fb, acc);
+                const float* q0 = box + (ib[0] - bx.lx) + (ib[1] - bx.ly) * pitch + (ib[2] - bx.lz) * sz;
+                if (pitch == kTmaX) gather_samples<kTmaX, kPlainBox, false>(r, box, q0, sz, j0, j1, fb, acc);
+                else if (pitch == 33) gather_samples<33, kPlainBox, false>(r, box, q0, sz, j0, j1, fb, acc);
+                else gather_samples<65, kPlainBox, false>(r, box, q0, sz, j0, j1, fb, acc);
             }
         } else if (act) {
             // the staged loop's own positions and blend, so that every path
@@ -152,7 +201,6 @@ __global__ void __launch_bounds__(RPB, 1024 / RPB) k_project(GridD g, int nu, in
 // wait is bounded (about one second of clock): a CTA that gives up counts
 // PMF_DIAG_TIMEOUT, waits once more for its copies, writes NaN to its pixels
 // and returns.
-constexpr int kTmaX = 44;                     // floats per staged row (one copy's x extent)
 constexpr int kTmaRows = 8;                   // rows per copy
 constexpr int kTmaSkew = 16;                  // extra plane stride (floats) of the conflict-free layout
 constexpr int kTmaBox = 13312;                // staged floats (52 KB of dynamic shared memory)
@@ -277,31 +325,8 @@ __device__ __forceinline__ bool project_tile_tma(const GridD& g, int nu, int nv,
                 return false;
             }
             if (act) {
-                const float syf = (float)kTmaX, szf = (float)S;
-                const int sy = kTmaX, sz = S;
-                const float* qa = box + (ib[0] - x0) + (ib[1] - bx.ly) * sy + (ib[2] - bx.lz) * sz;
-                // the staged loop's arithmetic with the x/y position and the
-                // z-paired blends in packed fp32 pairs (same bits, fewer
-                // instructions): (a00, a01), (a10, a11), then (b0, b1)
-                const f32x2 dxy = pack2(r.dh[0], r.dh[1]), bxy = pack2(fb[0], fb[1]), one = pack2(1.0f, 1.0f);
-                f32x2 jj = pack2((float)j0, (float)j0);
-#pragma unroll 2  // two samples' dependency chains interleave (measured 2% faster)
-                for (int j = j0; j <= j1; j++, jj = add2(jj, one)) {
-                    const f32x2 uxy = fma2(jj, dxy, bxy);
-                    const float ux = lo2(uxy), uy = hi2(uxy), uz = fmaf(lo2(jj), r.dh[2], fb[2]);
-                    const float flx = floorf(ux), fly = floorf(uy), flz = floorf(uz);
-                    const f32x2 fxy = sub2(uxy, pack2(flx, fly));
-                    const float fx = lo2(fxy), fy = hi2(fxy), fz = uz - flz;
-                    const float* q = qa + (int)fmaf(flz, szf, fmaf(fly, syf, flx));
-                    if (!PMF_DCHECK(q >= box && q + sz + sy + 1 < box + kTmaBox)) continue;
-                    const f32x2 c00 = pack2(q[0], q[sz]), c10 = pack2(q[1], q[sz + 1]);
-                    const f32x2 c01 = pack2(q[sy], q[sz + sy]), c11 = pack2(q[sy + 1], q[sz + sy + 1]);
-                    const f32x2 fx2 = pack2(fx, fx);
-                    const f32x2 a0 = fma2(fx2, sub2(c10, c00), c00), a1 = fma2(fx2, sub2(c11, c01), c01);
-                    const f32x2 bb = fma2(pack2(fy, fy), sub2(a1, a0), a0);
-                    const float b0 = lo2(bb), b1 = hi2(bb);
-                    acc += fmaf(fz, b1 - b0, b0);
-                }
+                const float* q0 = box + (ib[0] - x0) + (ib[1] - bx.ly) * kTmaX + (ib[2] - bx.lz) * S;
+                gather_samples<kTmaX, kTmaBox, true>(r, box, q0, S, j0, j1, fb, acc);
             }
         } else if (act) {
             // the staged loop's own positions and blend, so that every path
