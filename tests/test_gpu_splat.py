@@ -155,3 +155,26 @@ def test_rasterize_paper_scale_gradients(paper):
                                 wl.ref.value[sel], host(dY), wl.kappa)
     for name, a, b in zip(("mean", "scale", "quat", "value"), grads, ref):
         assert rel_l2(host(a)[sel].reshape(b.shape), b) <= TOLG, name
+
+
+@pytest.mark.parametrize("nu", [37, 40])
+def test_rasterize_adjoint_run_blocks(nu):
+    """The adjoint lists a row's pixel run in blocks of eight, from a multiple of
+    four with 16-byte image rows (nu = 40) and from the run's first pixel without
+    (37): runs of one pixel to the whole row, Gaussians far narrower than a
+    pixel (whose exponential three pixels out underflows) and wider than the
+    detector.  Both detectors against the oracle, with the forward's blocks."""
+    grid = Grid(24, 20, 16, 2.0, 2.0, 2.0)
+    rng = np.random.default_rng(61)
+    gs = gaussian_set(rng, grid, 60, 0.5, 3.0)
+    gs.scale[:20] = np.float32(0.05)  # 0.05 mm: a few hundredths of a pixel
+    gs.scale[20:24] = np.float32(40.0)  # wider than the detector
+    vw = circular_views(2, 300.0, 450.0, nu, 29, 1.4, 1.4, start=0.4)
+    det = Detector(nu, 29, 1.0)
+    Y = pmf.gs_rasterize(det, views(vw), gset(gs, 3.0))
+    assert rel_l2(host(Y), _oracle(det, vw, gs, 3.0)) <= TOL32
+    dY = rng.normal(size=(2, 29, nu)).astype(np.float32)
+    got = pmf.gs_rasterize_backward(det, views(vw), gset(gs, 3.0), dev(dY))
+    ref = oracle.splat_backward(det.nu, det.nv, vw, gs.mean, gs.scale, gs.quat, gs.value, dY, 3.0)
+    for name, a, b in zip(("mean", "scale", "quat", "value"), got, ref):
+        assert rel_l2(host(a), np.asarray(b).reshape(tuple(a.shape))) <= TOLG, name
