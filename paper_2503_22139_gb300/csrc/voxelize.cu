@@ -669,6 +669,21 @@ __device__ __forceinline__ float warp_sum(float r) {
     return r;
 }
 
+// The C + 9 moments of Gaussian i's slab, summed over the warp in a fixed tree.
+template <int C>
+__device__ __forceinline__ void item_moments(const pmf_gaussians& G, int64_t i, const GaussSetup& st, const GridD& g,
+                                             const float* __restrict__ dout, int slab, int S, bool vec, WarpPlan& plan,
+                                             float r[C + kMom]) {
+    Moments<C> m;
+    warp_moments<C>(G, i, st, g, dout, slab, S, vec, plan, m);
+#pragma unroll
+    for (int c = 0; c < C; c++) r[c] = warp_sum(m.gv[c]);
+#pragma unroll
+    for (int a = 0; a < 3; a++) r[C + a] = warp_sum(m.s1[a]);
+#pragma unroll
+    for (int a = 0; a < 6; a++) r[C + 3 + a] = warp_sum(m.s2[a]);
+}
+
 // Gradients of one Gaussian from its summed moments (thread-local).
 template <int C>
 __device__ void moments_to_grad(const GaussSetup& s, const float* r, int64_t i, float* d_mean, float* d_scale,
@@ -740,21 +755,52 @@ __global__ void __launch_bounds__(32 * kBwdItemWarps, (C == 1 ? 32 : 24) / kBwdI
     }
     __shared__ WarpPlan plan;
     static_assert(kBwdItemWarps == 1, "one plan per CTA");
-    Moments<C> m;
-    warp_moments<C>(G, i, st, g, dout, slab, S, vec, plan, m);
     float r[C + kMom];
-#pragma unroll
-    for (int c = 0; c < C; c++) r[c] = warp_sum(m.gv[c]);
-#pragma unroll
-    for (int a = 0; a < 3; a++) r[C + a] = warp_sum(m.s1[a]);
-#pragma unroll
-    for (int a = 0; a < 6; a++) r[C + 3 + a] = warp_sum(m.s2[a]);
+    item_moments<C>(G, i, st, g, dout, slab, S, vec, plan, r);
     if ((threadIdx.x & 31) != 0) return;
     if (S == 1) {
         moments_to_grad<C>(st, r, i, d_mean, d_scale, d_quat, d_value, accumulate);
     } else {
 #pragma unroll
         for (int k = 0; k < C + kMom; k++) part[item * (C + kMom) + k] = r[k];
+    }
+}
+
+// The same for one slab per Gaussian and a grid with fewer voxels than a few per
+// Gaussian -- a crop, most of the set outside it: a warp takes eight Gaussians, each
+// lane finds one's voxel box, the empty ones' zero gradients are written by their
+// own lanes, and the warp walks the others one after the other.  (100,000
+// Gaussians, a 32^3 crop: a warp per Gaussian took 62 us, nearly all of it warps
+// that return at once; a Stage-1 step 483 -> 455 us.  On a whole volume the walk's
+// registers spill and cost a tenth, so that stays with a warp per Gaussian.)
+constexpr int kSparsePer = 8;
+
+template <int C>
+__global__ void __launch_bounds__(32, C == 1 ? 32 : 24) k_vox_bwd_sparse(pmf_gaussians G, GridD g,
+                                                                         const float* __restrict__ dout, float* d_mean,
+                                                                         float* d_scale, float* d_quat, float* d_value,
+                                                                         int accumulate, bool vec) {
+    __shared__ WarpPlan plan;
+    const int lane = threadIdx.x & 31;
+    const int64_t first = (int64_t)blockIdx.x * kSparsePer, mine = first + lane;
+    bool full = false;
+    if (lane < kSparsePer && mine < G.n) {
+        GaussSetup st;
+        gauss_setup(G, mine, g, G.kappa, st);
+        full = st.lo[0] <= st.hi[0] && st.lo[1] <= st.hi[1] && st.lo[2] <= st.hi[2];
+        if (!full && !accumulate) {
+            for (int a = 0; a < 3; a++) d_mean[3 * mine + a] = d_scale[3 * mine + a] = 0.0f;
+            for (int a = 0; a < 4; a++) d_quat[4 * mine + a] = 0.0f;
+            for (int c = 0; c < C; c++) d_value[mine * C + c] = 0.0f;
+        }
+    }
+    for (unsigned todo = __ballot_sync(0xffffffffu, full); todo; todo &= todo - 1) {
+        const int64_t i = first + __ffs(todo) - 1;
+        GaussSetup st;
+        gauss_setup(G, i, g, G.kappa, st);
+        float r[C + kMom];
+        item_moments<C>(G, i, st, g, dout, 0, 1, vec, plan, r);
+        if (lane == 0) moments_to_grad<C>(st, r, i, d_mean, d_scale, d_quat, d_value, accumulate);
     }
 }
 
@@ -982,8 +1028,11 @@ pmf_status gs_voxelize_backward(const pmf_grid* grid, const pmf_gaussians* gs, c
     const unsigned nb = (unsigned)((items + kBwdItemWarps - 1) / kBwdItemWarps);
     const unsigned nf = (unsigned)((gs->n + kBwdWarps - 1) / kBwdWarps);
     const int T = 32 * kBwdWarps, TI = 32 * kBwdItemWarps;
+    const unsigned ns = (unsigned)((gs->n + kSparsePer - 1) / kSparsePer);
+    const bool sparse = S == 1 && g.n < 4 * gs->n;
 #define PMF_VB(CC)                                                                                               \
-    k_vox_bwd<CC><<<nb, TI, 0, s>>>(*gs, g, S, d_out, part, d_mean, d_scale, d_quat, d_value, accumulate, vec); \
+    if (sparse) k_vox_bwd_sparse<CC><<<ns, 32, 0, s>>>(*gs, g, d_out, d_mean, d_scale, d_quat, d_value, accumulate, vec); \
+    else k_vox_bwd<CC><<<nb, TI, 0, s>>>(*gs, g, S, d_out, part, d_mean, d_scale, d_quat, d_value, accumulate, vec); \
     if (S > 1) k_vox_bwd_final<CC><<<nf, T, 0, s>>>(*gs, g, S, part, d_mean, d_scale, d_quat, d_value, accumulate);
     switch (gs->channels) {
         case 1: { PMF_VB(1) break; }

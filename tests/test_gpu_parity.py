@@ -632,3 +632,25 @@ def test_voxelize_backward_row_plans(n, G, scale, C):
     ref = oracle.voxelize_backward(grid, gs.mean, gs.scale, gs.quat, gs.value, d, 3.0)
     for x, r in zip(got, ref):
         assert rel_l2(host(x), np.asarray(r).reshape(tuple(x.shape))) <= 1e-4
+
+
+@pytest.mark.parametrize("C", [1, 3])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_voxelize_backward_of_a_crop(C, accumulate):
+    """More Gaussians than the slabs' limit on a grid of fewer than four voxels
+    per Gaussian takes eight Gaussians per warp: those outside the grid get zero
+    (or nothing added), a sample of the others matches the oracle."""
+    grid = Grid(17, 16, 15, 2.0, 2.0, 2.0)
+    n = 20011  # above the slab limit of 152 * 64 * 4 / 2 warps, not a multiple of eight
+    gs = _rand_gaussians(430, grid, n, 1.0, 4.0, C)
+    gs.mean[::3] += np.float32(400.0)  # outside
+    g = gset(gs, 3.0)
+    d = dev(np.random.default_rng(431).normal(size=(C,) + grid.shape))
+    base = [torch.full(s, 0.25, device="cuda") for s in ((n, 3), (n, 3), (n, 4), (n, C))]
+    got = pmf.gs_voxelize_backward(grid, g, d, grads=tuple(base) if accumulate else None, accumulate=accumulate)
+    for x in got:
+        assert torch.all(x[::3] == (0.25 if accumulate else 0.0))
+    sel = np.arange(1, n, 1500)
+    ref = oracle.voxelize_backward(grid, gs.mean[sel], gs.scale[sel], gs.quat[sel], gs.value[sel], host(d), 3.0)
+    for x, r in zip(got, ref):
+        assert rel_l2(host(x)[sel] - (0.25 if accumulate else 0.0), np.asarray(r).reshape(len(sel), -1)) <= 1e-4
