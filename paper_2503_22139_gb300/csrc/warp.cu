@@ -546,8 +546,8 @@ __device__ __forceinline__ void stage_halo_pairs(const T* __restrict__ ref, cons
 template <class G>
 __device__ __forceinline__ void corners8_pairs(const float2* sv2, int rx, int ry, int rz, float cv[8]) {
     constexpr int SY = G::PX, SZ = G::PX * G::BY;
-    const int r0 = rz * G::BY + ry;  // rows of the cell's y and y + 1 corners (and +BY for z + 1)
-    const int i0 = r0 * SY + pair_col<G>(rx, r0), i1 = (r0 + 1) * SY + pair_col<G>(rx, r0 + 1);
+    const int r0 = rz * G::BY + ry;  // row of the cell's lower corner (+1 for y + 1, +BY for z + 1)
+    const int i0 = r0 * SY + pair_col<G>(rx, r0), i1 = (i0 ^ 8) + SY;  // the next row's rotation is the other one
     if (!PMF_DCHECK(i0 >= 0 && i1 >= 0 && i0 + SZ < G::BOXN && i1 + SZ < G::BOXN)) {
 #pragma unroll
         for (int c = 0; c < 8; c++) cv[c] = 0.0f;
