@@ -158,6 +158,7 @@ def forward_model(grid, det, ref: Sequence[torch.Tensor], mbc: Sequence[Sequence
     Returns (Y, loss) with loss None when `meas` is None.  kind "eq14": the
     objective of Eq. 14 (eq14 = dict(lambda_ssim, lambda_mbc, lambda_tv,
     data_range, tv_size, tv_origin))."""
+    grid, det = ops._grid(grid), ops._det(det)  # converted once for all calls
     V = voxelize(grid, *ref, kappa=kappa, dtype=dtype)[0]
     E = torch.stack([voxelize(grid, *m, kappa=kappa, dtype=dtype) for m in mbc])
     W = warp_combine(grid, V, E, coeff)

@@ -23,6 +23,8 @@ _DT = {torch.float32: 0, torch.bfloat16: 1, torch.float16: 2}
 
 
 def _grid(g) -> PmfGrid:
+    if type(g) is PmfGrid:
+        return g
     if hasattr(g, "nx"):
         return PmfGrid(int(g.nx), int(g.ny), int(g.nz), float(g.vx), float(g.vy), float(g.vz))
     nx, ny, nz, vx, vy, vz = g
@@ -30,6 +32,8 @@ def _grid(g) -> PmfGrid:
 
 
 def _det(d) -> PmfDetector:
+    if type(d) is PmfDetector:
+        return d
     if hasattr(d, "nu"):
         return PmfDetector(int(d.nu), int(d.nv), float(d.step_mm))
     nu, nv, step = d
@@ -42,7 +46,9 @@ def _shape(g):
 
 
 def _stream():
-    return ct.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the current stream's handle itself: building a torch.cuda.Stream around it
+    # took about 10 us of each call
+    return ct.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _p(t: Optional[torch.Tensor]):
@@ -122,19 +128,33 @@ def gs_voxelize_count(grid, gs: Gaussians, tile=None) -> int:
     return int(out.item())
 
 
+# Lists of up to this many pairs (16 MB) are allocated at their bound.
+_BOUND_PAIRS = 1 << 22
+
+
+def _pair_capacity(g: PmfGrid, gs: Gaussians, tile=None) -> int:
+    """List capacity of a call without a workspace: the bound n x tiles where
+    that is small, else the exact count.  Counting launches the set-up twice and
+    waits for the GPU, which a small set's call (a few dozen us of kernels)
+    spends most of its time on; the list holds the same pairs either way."""
+    tx, ty, tz = (int(t) for t in (tile or VOXEL_TILES[0]))
+    bound = gs.n * (-(-g.nx // tx)) * (-(-g.ny // ty)) * (-(-g.nz // tz))
+    return bound if bound <= _BOUND_PAIRS else gs_voxelize_count(g, gs, tile)
+
+
 def gs_voxelize(grid, gs: Gaussians, dtype=torch.float32, pair_capacity: Optional[int] = None,
                 out: Optional[torch.Tensor] = None, ws: Optional[torch.Tensor] = None, tile=None) -> torch.Tensor:
     """Eq. 5 / signed MBC voxelization -> [C, nz, ny, nx] of `dtype`; tile: the
     bin tile (one of VOXEL_TILES; the default 8^3 calls gs_voxelize itself)."""
     L = _lib.load()
     g = _grid(grid)
-    shape, n = _shape(grid)
+    shape, n = _shape(g)
     dev = gs.mean.device
     if out is None:
         out = torch.empty((gs.channels,) + shape, dtype=dtype, device=dev)
     if ws is None:
-        cap = gs_voxelize_count(grid, gs, tile) if pair_capacity is None else int(pair_capacity)
-        ws = _ws(gs_voxelize_workspace(grid, gs.n, cap, tile), dev)
+        cap = _pair_capacity(g, gs, tile) if pair_capacity is None else int(pair_capacity)
+        ws = _ws(gs_voxelize_workspace(g, gs.n, cap, tile), dev)
     s = gs.c_struct()
     if tile is None:
         check(L.gs_voxelize(ct.byref(g), ct.byref(s), _DT[out.dtype], _p(out), _p(ws), ws.numel(), _stream()),
@@ -170,7 +190,7 @@ def gs_voxelize_backward(grid, gs: Gaussians, d_out: torch.Tensor, grads=None, a
         grads = (torch.empty((gs.n, 3), device=dev), torch.empty((gs.n, 3), device=dev),
                  torch.empty((gs.n, 4), device=dev), torch.empty((gs.n, gs.channels), device=dev))
     if ws is None:
-        ws = _ws(gs_voxelize_backward_workspace(grid, gs.n, gs.channels), dev)
+        ws = _ws(gs_voxelize_backward_workspace(g, gs.n, gs.channels), dev)
     s = gs.c_struct()
     check(L.gs_voxelize_backward(ct.byref(g), ct.byref(s), _p(d_out), *[_p(t) for t in grads], int(accumulate),
                                  _p(ws), ws.numel(), _stream()), "gs_voxelize_backward")
@@ -298,6 +318,7 @@ def mbc_combine(grid, mbc: torch.Tensor, coeff: torch.Tensor, out=None) -> torch
     mbc = _need(mbc, "mbc")
     coeff = _need(coeff, "coeff", torch.float32)
     P, Lv = int(coeff.shape[0]), int(coeff.shape[1])
+    grid = _grid(grid)
     shape, n = _shape(grid)
     if out is None:
         out = torch.empty((P, 3) + shape, dtype=mbc.dtype, device=mbc.device)
@@ -373,6 +394,7 @@ def warp_combine(grid, ref, mbc, coeff, out=None) -> torch.Tensor:
     ref, mbc = _need(ref, "ref"), _need(mbc, "mbc")
     coeff = _need(coeff, "coeff", torch.float32)
     P, Lv = int(coeff.shape[0]), int(coeff.shape[1])
+    grid = _grid(grid)
     shape, _ = _shape(grid)
     if out is None:
         out = torch.empty((P,) + shape, dtype=ref.dtype, device=ref.device)
@@ -450,6 +472,7 @@ def conebeam_project(grid, det, views: torch.Tensor, vol: torch.Tensor, shared: 
     views = _need(views, "views", torch.float64)
     P = int(views.shape[0])
     d = _det(det)
+    grid = _grid(grid)
     _, n = _shape(grid)
     if shared is None:
         shared = vol.numel() == n
@@ -472,7 +495,7 @@ def conebeam_project_backward(grid, det, views, d_proj, shared: bool = False, ac
     P = int(views.shape[0])
     d = _det(det)
     g = _grid(grid)
-    shape, n = _shape(grid)
+    shape, n = _shape(g)
     stride = 0 if shared else n
     if ws is None:
         ws = _ws(_size(L.conebeam_project_backward_workspace, ct.byref(g), P, stride), d_proj.device)

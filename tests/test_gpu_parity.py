@@ -654,3 +654,17 @@ def test_voxelize_backward_of_a_crop(C, accumulate):
     ref = oracle.voxelize_backward(grid, gs.mean[sel], gs.scale[sel], gs.quat[sel], gs.value[sel], host(d), 3.0)
     for x, r in zip(got, ref):
         assert rel_l2(host(x)[sel] - (0.25 if accumulate else 0.0), np.asarray(r).reshape(len(sel), -1)) <= 1e-4
+
+
+@pytest.mark.parametrize("G", [0, 1, 40])
+def test_voxelize_without_workspace_takes_the_pair_bound(G):
+    """A small call without a workspace allocates the list's bound, n x tiles,
+    instead of counting: the same bits as with the exact count, whose value the
+    bound covers."""
+    grid = Grid(21, 17, 9, 2.0, 2.0, 2.0)
+    gs = gset(_rand_gaussians(440, grid, max(G, 1), 1.0, 5.0, 3), 3.0)
+    if G == 0:
+        gs = pmf.Gaussians(gs.mean[:0], gs.scale[:0], gs.quat[:0], gs.value[:0], 3.0)
+    exact = pmf.gs_voxelize_count(grid, gs)
+    assert exact <= pmf.ops._pair_capacity(pmf.ops._grid(grid), gs) == G * 3 * 3 * 2
+    assert torch.equal(pmf.gs_voxelize(grid, gs), pmf.gs_voxelize(grid, gs, pair_capacity=exact))
