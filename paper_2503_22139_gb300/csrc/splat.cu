@@ -423,15 +423,13 @@ __device__ __forceinline__ float warp_allsum(float v) {
 // 8 pixels, and the six sums
 //   sum dY e,  sum c (K d)_a,  sum c (K d)_b,  sum c d_a^2,  sum c d_a d_b,  sum c d_b^2
 // (c = dY rho^ e, d = x^ - p^) accumulate per lane; a fixed butterfly reduces
-// them and lane 0 writes them to sums[view][Gaussian].
-// Bound by the L1 wavefronts of its loads (32 rows a load): where image rows are
-// 16-byte multiples the blocks start at a multiple of four pixels and their dY
-// come by two 16-byte loads (a Stage-1 step 466 -> 455 us).  Dealing the runs'
-// blocks to the lanes by a warp scan, as the voxelizer's adjoint does, evened the
-// lanes out but cost as much as it saved (162 us a view against 155).
+// them and lane 0 writes them to sums[view][Gaussian].  L1 wavefronts bind it (76%
+// of their peak, 32 rows a load).  Tried and slower: the dY of aligned blocks by
+// two 16-byte loads (LSU 36%, but masked first pixels: 644 us against 568 for four
+// views), and the runs' blocks dealt to the lanes by a warp scan (162 against 155 a
+// view).
 __global__ void __launch_bounds__(32 * kBwdWarps, 4) k_splat_bwd_sums(int64_t n, int P, int nu, int nv, float kappa,
-                                                                   RasterWs w, const float* __restrict__ dproj,
-                                                                   bool vec) {
+                                                                   RasterWs w, const float* __restrict__ dproj) {
     const int64_t pair = (int64_t)blockIdx.x * kBwdWarps + (threadIdx.x >> 5);
     if (pair >= (int64_t)P * n) return;  // whole warps
     const int lane = threadIdx.x & 31;
@@ -472,30 +470,20 @@ __global__ void __launch_bounds__(32 * kBwdWarps, 4) k_splat_bwd_sums(int64_t n,
             const float* row = dp + (int64_t)j * nu;
             // the carried products drift by about k^2/2 ulps after k steps: restart
             // them from exact values every 8 pixels
-            for (int ib = vec ? i0 & ~3 : i0; ib <= i1; ib += 8) {
+            for (int ib = i0; ib <= i1; ib += 8) {
                 // the block's dY values are loaded before any is used, so the
                 // (L2-latency) loads of a block overlap
+                const int cnt = min(i1 - ib, 7);
                 float gyb[8];
-                if (vec) {  // whole 16-byte groups of the row: ib and nu are multiples of four
-                    const float4 u0 = __ldg(reinterpret_cast<const float4*>(row + ib));
-                    const float4 u1 = ib + 4 <= i1 ? __ldg(reinterpret_cast<const float4*>(row + ib + 4))
-                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
-                    gyb[0] = u0.x; gyb[1] = u0.y; gyb[2] = u0.z; gyb[3] = u0.w;
-                    gyb[4] = u1.x; gyb[5] = u1.y; gyb[6] = u1.z; gyb[7] = u1.w;
-                } else {
 #pragma unroll
-                    for (int k = 0; k < 8; k++) gyb[k] = ib + k <= i1 ? __ldg(row + ib + k) : 0.0f;
-                }
-                // from the block's first pixel in the run: a narrow Gaussian's e
-                // three pixels outside would underflow
-                float da = pixel_x(max(ib, i0), nu) - rc.a;
+                for (int k = 0; k < 8; k++) gyb[k] = k <= cnt ? __ldg(row + ib + k) : 0.0f;
+                float da = pixel_x(ib, nu) - rc.a;
                 float e = __expf(-0.5f * splat_q(rc.k0, rc.k1, rc.k2, da, db));
                 float r = __expf(-fmaf(rc.k0, da + 0.5f, hb));
                 float ka = fmaf(rc.k0, da, hb), kb = fmaf(rc.k1, da, kbd);
 #pragma unroll
                 for (int k = 0; k < 8; k++) {
-                    if (ib + k < i0) continue;
-                    if (ib + k > i1) break;
+                    if (k > cnt) break;
                     const float gy = gyb[k];
                     const float ge = gy * e, c = ge * rc.rho, cd = c * da;
                     s0 += ge;
@@ -742,7 +730,7 @@ pmf_status gs_rasterize_backward(const pmf_detector* det, int32_t P, const pmf_v
     const int64_t pairs = (int64_t)P * g->n;
     if (pairs > 0)
         k_splat_bwd_sums<<<(unsigned)((pairs + kBwdWarps - 1) / kBwdWarps), 32 * kBwdWarps, 0, s>>>(
-            g->n, P, det->nu, det->nv, g->kappa, w, d_proj, det->nu % 4 == 0 && ((uintptr_t)d_proj & 15) == 0);
+            g->n, P, det->nu, det->nv, g->kappa, w, d_proj);
     k_splat_bwd_chain<<<(unsigned)((g->n + 127) / 128), 128, 0, s>>>(*g, P, w, d_mean, d_scale, d_quat, d_value,
                                                                     accumulate);
     return check_launch("gs_rasterize_backward");

@@ -159,11 +159,10 @@ def test_rasterize_paper_scale_gradients(paper):
 
 @pytest.mark.parametrize("nu", [37, 40])
 def test_rasterize_adjoint_run_blocks(nu):
-    """The adjoint lists a row's pixel run in blocks of eight, from a multiple of
-    four with 16-byte image rows (nu = 40) and from the run's first pixel without
-    (37): runs of one pixel to the whole row, Gaussians far narrower than a
-    pixel (whose exponential three pixels out underflows) and wider than the
-    detector.  Both detectors against the oracle, with the forward's blocks."""
+    """The render's and the adjoint's pixel blocks at their extremes: runs of one
+    pixel to the whole row, Gaussians far narrower than a pixel (whose
+    exponential a few pixels out underflows) and wider than the detector, on
+    image rows that are and are not 16-byte multiples, against the oracle."""
     grid = Grid(24, 20, 16, 2.0, 2.0, 2.0)
     rng = np.random.default_rng(61)
     gs = gaussian_set(rng, grid, 60, 0.5, 3.0)
