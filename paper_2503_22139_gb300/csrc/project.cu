@@ -68,6 +68,8 @@ __device__ __forceinline__ void gather_samples(const Ray& r, const float* box, c
 // latter, with 1.3 wavefronts per load, and a scalar blend: four fp32 volumes of
 // odd sizes, 16 views, both ways: 3,565 -> 3,390 us.)
 __device__ __forceinline__ int plain_layout(const Box& bx, int& sz) {
+    sz = 0;
+    if (bx.by > kPlainBox) return 0;
     sz = bx.by * kTmaX;
     sz += (16 - sz) & 31;
     if (bx.bx <= kTmaX && (long long)bx.bz * sz <= kPlainBox) return kTmaX;

@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(32 * kBwdItemWarps, (C == 1 ? 32 : 24) / kBwdI
 // lane finds one's voxel box, the empty ones' zero gradients are written by their
 // own lanes, and the warp walks the others one after the other.  (100,000
 // Gaussians, a 32^3 crop: a warp per Gaussian took 62 us, nearly all of it warps
-// that return at once; a Stage-1 step 483 -> 455 us.  On a whole volume the walk's
+// that return at once; 28 us so.  On a whole volume the walk's
 // registers spill and cost a tenth, so that stays with a warp per Gaussian.)
 constexpr int kSparsePer = 8;
 
