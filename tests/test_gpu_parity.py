@@ -668,3 +668,25 @@ def test_voxelize_without_workspace_takes_the_pair_bound(G):
     exact = pmf.gs_voxelize_count(grid, gs)
     assert exact <= pmf.ops._pair_capacity(pmf.ops._grid(grid), gs) == G * 3 * 3 * 2
     assert torch.equal(pmf.gs_voxelize(grid, gs), pmf.gs_voxelize(grid, gs, pair_capacity=exact))
+
+
+def test_voxelize_backward_on_a_grid_of_2_31_rows():
+    """A grid one voxel wide whose last rows have an index past 2^31 (8.6 GB of
+    upstream gradient): a Gaussian at that corner gets the gradient of the same
+    Gaussian on a 41 x 41 patch with the same voxel centres (both axes odd, 1 mm
+    voxels: every centre and difference is exact), within the bound used above."""
+    n, m = 46401, 41
+    grid, patch = Grid(1, n, n, 1.0, 1.0, 1.0), Grid(1, m, m, 1.0, 1.0, 1.0)
+    assert (n - m) * n >= 2 ** 31
+    d = np.random.default_rng(450).normal(size=(1, m, m, 1)).astype(np.float32)
+    d_big = torch.zeros((1, n, n, 1), dtype=torch.float32, device="cuda")
+    d_big[:, n - m:, n - m:] = dev(d)
+    gs = gaussian_set(np.random.default_rng(451), patch, 1, 2.0, 3.0, channels=1)
+    gs.mean[0] = (0.0, 0.25, -0.5)
+    centre = (n - m) // 2  # the patch's centre voxel in the grid, mm from its own centre
+    big = gset(gs, 3.0)
+    big.mean[0, 1:] += float(centre)
+    got = pmf.gs_voxelize_backward(grid, big, d_big)
+    ref = oracle.voxelize_backward(patch, gs.mean, gs.scale, gs.quat, gs.value, d, 3.0)
+    for x, r in zip(got, ref):
+        assert rel_l2(host(x), np.asarray(r).reshape(tuple(x.shape))) <= 1e-4
