@@ -136,7 +136,10 @@ def _pair_capacity(g: PmfGrid, gs: Gaussians, tile=None) -> int:
     """List capacity of a call without a workspace: the bound n x tiles where
     that is small, else the exact count.  Counting launches the set-up twice and
     waits for the GPU, which a small set's call (a few dozen us of kernels)
-    spends most of its time on; the list holds the same pairs either way."""
+    spends most of its time on; the list holds the same pairs either way.  A tile
+    that is none of VOXEL_TILES goes to the count, which refuses it."""
+    if tile is not None and tuple(int(t) for t in tile) not in VOXEL_TILES:
+        return gs_voxelize_count(g, gs, tile)
     tx, ty, tz = (int(t) for t in (tile or VOXEL_TILES[0]))
     bound = gs.n * (-(-g.nx // tx)) * (-(-g.ny // ty)) * (-(-g.nz // tz))
     return bound if bound <= _BOUND_PAIRS else gs_voxelize_count(g, gs, tile)

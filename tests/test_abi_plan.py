@@ -6,6 +6,7 @@ before any CUDA call."""
 import ctypes as ct
 import os
 import subprocess
+import types
 
 import numpy as np
 import pytest
@@ -173,3 +174,13 @@ def test_plan_rejects_incomplete_eq14_descriptors():
         h = ct.c_void_p(0)
         assert L.pmf_plan_create(ct.byref(d), ct.byref(h)) == -1
         assert msg in L.pmf_last_error()
+
+
+@pytest.mark.parametrize("tile", [(0, 8, 8), (8, 8, 0), (4, 4, 4), (8, 8)])
+def test_pair_capacity_refuses_unsupported_tiles(tile):
+    """A call without a workspace sizes its list on the host before the library
+    sees the tile: one that the library does not support gets the library's
+    error, whatever the set's size (a zero extent was a ZeroDivisionError)."""
+    gs = types.SimpleNamespace(n=5, mean=types.SimpleNamespace(device="cpu"))
+    with pytest.raises(_lib.PmfError, match="not supported"):
+        ops._pair_capacity(ops._grid((16, 16, 16, 2.0, 2.0, 2.0)), gs, tile)
