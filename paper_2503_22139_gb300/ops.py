@@ -46,9 +46,13 @@ def _shape(g):
 
 
 def _stream():
-    # the current stream's handle itself: building a torch.cuda.Stream around it
-    # took about 10 us of each call
-    return ct.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    # the current stream's handle itself (building a torch.cuda.Stream around it
+    # takes about 10 us of each call) where torch has the call for it, which is
+    # not part of its public interface
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return ct.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return ct.c_void_p(raw(torch.cuda.current_device()))
 
 
 def _p(t: Optional[torch.Tensor]):

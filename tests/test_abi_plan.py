@@ -10,6 +10,7 @@ import types
 
 import numpy as np
 import pytest
+import torch
 
 import paper_2503_22139_gb300.ops as ops
 from paper_2503_22139_gb300 import _lib
@@ -184,3 +185,11 @@ def test_pair_capacity_refuses_unsupported_tiles(tile):
     gs = types.SimpleNamespace(n=5, mean=types.SimpleNamespace(device="cpu"))
     with pytest.raises(_lib.PmfError, match="not supported"):
         ops._pair_capacity(ops._grid((16, 16, 16, 2.0, 2.0, 2.0)), gs, tile)
+
+
+def test_stream_handle_without_the_private_torch_call(monkeypatch):
+    """torch's raw-stream call is not public: without it the handle comes from
+    the current stream's object."""
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0x1234))
+    assert ops._stream().value == 0x1234
