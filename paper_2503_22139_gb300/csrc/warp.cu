@@ -235,48 +235,77 @@ __global__ void k_reduce_partials(const float* part, int64_t nout, int nb, float
 
 // --------------------------------------------------------------- warp
 
-// A CTA takes 32 x 8 voxels of kWarpZ planes of one view (a lane its kWarpZ
-// voxels of one column): the voxel's coordinates come from one 32-bit block
-// index, where the flat index cost three 64-bit divisions per voxel, and the
-// loads of a lane's voxels overlap.  At the paper grid, one fp32 view: 43 ->
-// 30 us (80 MB: 12 us at the copy rate).
-constexpr int kWarpZ = 2;
-
+// A CTA takes a tile of one view, X x 8 voxels of 32 / X groups of Z planes (a
+// lane its Z voxels of one column; a warp 32 / X rows of X voxels): the voxel's
+// coordinates come from one 32-bit block index, where the flat index cost three
+// 64-bit divisions per voxel, and the loads of a lane's voxels overlap.  At the
+// paper grid, one fp32 view: 43 -> 30 us (80 MB: 12 us at the copy rate).
 struct WarpTiles {
     unsigned ntx, nty, ntz;
+    int x, z;  // X and Z
     unsigned per_view() const { return ntx * nty * ntz; }
 };
 
-WarpTiles warp_tiles(const GridD& g) {
-    return WarpTiles{(unsigned)((g.nx + 31) / 32), (unsigned)((g.ny + 7) / 8), (unsigned)((g.nz + kWarpZ - 1) / kWarpZ)};
+// X is 32 where at least 85% of a row's tiles are voxels, else 16 where that
+// much of them is, else 8, so that a narrow or odd row does not leave a third of
+// the lanes and more idle: eight fp32 views, X = 32 against the choice, forward
+// and adjoint, 36 x 64 x 64 voxels (X = 8) 20.5 -> 16.4 and 56 -> 46 us, 161 x 160
+// x 80 (X = 16) 119 -> 116 and 325 -> 303, 8 x 200 x 100 (X = 8) 41 -> 16 and 105
+// -> 54; at 200 voxels, 89% full, X = 16 takes the forward from 215 to 228.
+// Z is 2 for the overlap, or 1 where that leaves the GPU below ten blocks an SM
+// and latency decides: one fp32 view of 48 x 48 x 24, forward 8.2 -> 6.8 us.
+WarpTiles warp_tiles(const GridD& g, int P) {
+    auto tiles = [&](int x, int z) {
+        const int depth = z * (32 / x);
+        return WarpTiles{(unsigned)((g.nx + x - 1) / x), (unsigned)((g.ny + 7) / 8),
+                         (unsigned)((g.nz + depth - 1) / depth), x, z};
+    };
+    int x = 32;
+    while (x > 8 && 100 * (int64_t)g.nx < 85 * (int64_t)x * ((g.nx + x - 1) / x)) x /= 2;
+    const WarpTiles t = tiles(x, 2);
+    return (int64_t)t.per_view() * P < 10 * 152 ? tiles(x, 1) : t;
 }
 
-// Views per launch, so that the block index stays below 2^31 (a view has at
-// most n / 2 blocks, on a grid one voxel wide and high).
+// The view and the first voxel of a thread.
+struct WarpVoxel {
+    unsigned p;
+    int i, j, k0;
+};
+
+template <int X, int Z>
+__device__ __forceinline__ WarpVoxel warp_voxel(const WarpTiles& nt) {
+    constexpr int R = 32 / X;  // rows of a warp, all in one group of planes
+    const unsigned b = blockIdx.x, bz = b / (nt.ntx * nt.nty), r = b - bz * (nt.ntx * nt.nty);
+    const unsigned p = bz / nt.ntz, tz = bz - p * nt.ntz, ty = r / nt.ntx, tx = r - ty * nt.ntx;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (R == 1) return WarpVoxel{p, (int)(tx * 32) + lane, (int)(ty * 8) + warp, (int)tz * Z};
+    return WarpVoxel{p, (int)(tx * X) + lane % X, (int)(ty * 8) + warp * R % 8 + lane / X, ((int)tz * R + warp * R / 8) * Z};
+}
+
+// Views per launch, so that the block index stays below 2^31 (a view has fewer
+// blocks than n / 4).
 int views_per_launch(const WarpTiles& nt) {
     const int64_t per = (((int64_t)1 << 31) - 1) / nt.per_view();
     return (int)(per > 0 ? per : 1);
 }
 
-template <typename T>
+template <typename T, int X, int Z>
 __global__ void __launch_bounds__(kThreads) k_warp(GridD g, WarpTiles nt, const T* __restrict__ ref,
                                                    const T* __restrict__ D, T* __restrict__ W) {
-    const unsigned b = blockIdx.x, bz = b / (nt.ntx * nt.nty), r = b - bz * (nt.ntx * nt.nty);
-    const unsigned p = bz / nt.ntz, tz = bz - p * nt.ntz, ty = r / nt.ntx, tx = r - ty * nt.ntx;
-    const int i = (int)(tx * 32 + (threadIdx.x & 31)), j = (int)(ty * 8 + (threadIdx.x >> 5)), k0 = (int)tz * kWarpZ;
+    const auto [p, i, j, k0] = warp_voxel<X, Z>(nt);
     if (i >= g.nx || j >= g.ny) return;
     const int64_t N = g.n;
     const T* Dp = D + (int64_t)p * 3 * N;
     T* Wp = W + (int64_t)p * N;
-    float d[kWarpZ][3];
+    float d[Z][3];
 #pragma unroll
-    for (int h = 0; h < kWarpZ; h++) {
+    for (int h = 0; h < Z; h++) {
         const int64_t v = ((int64_t)(k0 + h) * g.ny + j) * g.nx + i;
 #pragma unroll
         for (int c = 0; c < 3; c++) d[h][c] = k0 + h < g.nz ? Store<T>::ld(Dp, c * N + v) : 0.f;
     }
 #pragma unroll
-    for (int h = 0; h < kWarpZ; h++) {
+    for (int h = 0; h < Z; h++) {
         if (k0 + h >= g.nz) break;
         const int64_t v = ((int64_t)(k0 + h) * g.ny + j) * g.nx + i;
         const Cell c = make_cell(i, j, k0 + h, d[h][0] * g.ivx, d[h][1] * g.ivy, d[h][2] * g.ivz);
@@ -937,37 +966,36 @@ __global__ void __launch_bounds__(GeomBwd::THREADS, 2) k_wc_bwd_tile(GridD g, in
 // atomics are left of eight.  At the paper grid, one fp32 view: 78 -> 72 us.  (The
 // fused adjoint's shared-memory box was tried here: with one view per tile its
 // zeroing, staging and flush took 228 us, and 32-bit terms are less exact.)
-template <typename T>
+template <typename T, int X, int Z>
 __global__ void __launch_bounds__(kThreads) k_warp_bwd(GridD g, WarpTiles nt, const T* __restrict__ ref,
                                                        const T* __restrict__ D, const float* __restrict__ dW,
                                                        float* d_dvf, unsigned long long* acc, const unsigned* maxbits,
                                                        float bound_mult, int accumulate) {
-    const unsigned b = blockIdx.x, bz = b / (nt.ntx * nt.nty), r = b - bz * (nt.ntx * nt.nty);
-    const unsigned p = bz / nt.ntz, tz = bz - p * nt.ntz, ty = r / nt.ntx, tx = r - ty * nt.ntx;
+    const auto [p, i, j, k0] = warp_voxel<X, Z>(nt);
     const int lane = threadIdx.x & 31;
-    const int i = (int)tx * 32 + lane, j = (int)(ty * 8 + (threadIdx.x >> 5)), k0 = (int)tz * kWarpZ;
-    if (j >= g.ny) return;  // whole warps
+    const bool inxy = i < g.nx && j < g.ny;
+    if (!__any_sync(0xffffffffu, inxy)) return;
     const int64_t N = g.n;
     const T* Dp = D + (int64_t)p * 3 * N;
     const float* dWp = dW + (int64_t)p * N;
     const int kexp = fixed_exponent(__uint_as_float(*maxbits) * bound_mult);
     const float scale = ldexpf(1.0f, kexp);
-    float d[kWarpZ][3], gwv[kWarpZ];
+    float d[Z][3], gwv[Z];
 #pragma unroll
-    for (int h = 0; h < kWarpZ; h++) {
-        const bool in = i < g.nx && k0 + h < g.nz;
+    for (int h = 0; h < Z; h++) {
+        const bool in = inxy && k0 + h < g.nz;
         const int64_t v = ((int64_t)(k0 + h) * g.ny + j) * g.nx + i;
 #pragma unroll
         for (int c = 0; c < 3; c++) d[h][c] = in ? Store<T>::ld(Dp, c * N + v) : 0.f;
         gwv[h] = in ? __ldg(dWp + v) : 0.f;
     }
 #pragma unroll
-    for (int h = 0; h < kWarpZ; h++) {
+    for (int h = 0; h < Z; h++) {
         if (k0 + h >= g.nz) break;
         const int64_t v = ((int64_t)(k0 + h) * g.ny + j) * g.nx + i;
         const float gw = gwv[h];
         const Cell c = make_cell(i, j, k0 + h, d[h][0] * g.ivx, d[h][1] * g.ivy, d[h][2] * g.ivz);
-        if (d_dvf && i < g.nx) {
+        if (d_dvf && inxy) {
             float gx, gy, gz;
             trilin_grad(ref, g, c, gx, gy, gz);
             float* o = d_dvf + (int64_t)p * 3 * N + v;
@@ -1168,6 +1196,17 @@ void launch_wc_bwd(unsigned nt, size_t smem, cudaStream_t s, const GridD& g, int
                                                 part, accumulate);
 }
 
+// The tile's shape -> template instantiation.
+#define PMF_DISPATCH_WARP_TILE(nt, X, Z, ...)                                    \
+    switch ((nt).x + (nt).z) {                                                   \
+        case 9: { constexpr int X = 8, Z = 1; __VA_ARGS__; break; }              \
+        case 10: { constexpr int X = 8, Z = 2; __VA_ARGS__; break; }             \
+        case 17: { constexpr int X = 16, Z = 1; __VA_ARGS__; break; }            \
+        case 18: { constexpr int X = 16, Z = 2; __VA_ARGS__; break; }            \
+        case 33: { constexpr int X = 32, Z = 1; __VA_ARGS__; break; }            \
+        default: { constexpr int X = 32, Z = 2; __VA_ARGS__; break; }            \
+    }
+
 pmf_status check_common(const pmf_grid* grid, int32_t P, pmf_dtype dtype) {
     pmf_status st = validate_grid(grid);
     if (st != PMF_OK) return st;
@@ -1236,11 +1275,12 @@ pmf_status warp_volume(const pmf_grid* grid, int32_t P, pmf_dtype dtype, const v
     PMF_REQUIRE(ref && dvf && out, "null pointer");
     GridD g = make_grid(grid);
     cudaStream_t s = (cudaStream_t)stream;
-    const WarpTiles nt = warp_tiles(g);
+    const WarpTiles nt = warp_tiles(g, P);
     const int per = views_per_launch(nt);
     for (int p0 = 0; p0 < P; p0 += per) {
         const int np = P - p0 < per ? P - p0 : per;
-        PMF_DISPATCH_DTYPE(dtype, T, k_warp<T><<<nt.per_view() * (unsigned)np, kThreads, 0, s>>>(g, nt, (const T*)ref, (const T*)dvf + (int64_t)p0 * 3 * g.n, (T*)out + (int64_t)p0 * g.n));
+        PMF_DISPATCH_DTYPE(dtype, T, PMF_DISPATCH_WARP_TILE(nt, X, Z,
+            k_warp<T, X, Z><<<nt.per_view() * (unsigned)np, kThreads, 0, s>>>(g, nt, (const T*)ref, (const T*)dvf + (int64_t)p0 * 3 * g.n, (T*)out + (int64_t)p0 * g.n)));
     }
     return check_launch("warp_volume");
 }
@@ -1270,11 +1310,12 @@ pmf_status warp_volume_backward(const pmf_grid* grid, int32_t P, pmf_dtype dtype
     cudaMemsetAsync(ws, 0, need, s);
     if (P > 0) {
         k_absmax<<<stream_blocks(g.n * P), kThreads, 0, s>>>(d_out, g.n * P, maxbits);
-        const WarpTiles nt = warp_tiles(g);
+        const WarpTiles nt = warp_tiles(g, P);
         const int per = views_per_launch(nt);
         for (int p0 = 0; p0 < P; p0 += per) {
             const int np = P - p0 < per ? P - p0 : per;
-            PMF_DISPATCH_DTYPE(dtype, T, k_warp_bwd<T><<<nt.per_view() * (unsigned)np, kThreads, 0, s>>>(g, nt, (const T*)ref, (const T*)dvf + (int64_t)p0 * 3 * g.n, d_out + (int64_t)p0 * g.n, d_dvf ? d_dvf + (int64_t)p0 * 3 * g.n : nullptr, acc, maxbits, (float)(g.n * (int64_t)P), accumulate));
+            PMF_DISPATCH_DTYPE(dtype, T, PMF_DISPATCH_WARP_TILE(nt, X, Z,
+                k_warp_bwd<T, X, Z><<<nt.per_view() * (unsigned)np, kThreads, 0, s>>>(g, nt, (const T*)ref, (const T*)dvf + (int64_t)p0 * 3 * g.n, d_out + (int64_t)p0 * g.n, d_dvf ? d_dvf + (int64_t)p0 * 3 * g.n : nullptr, acc, maxbits, (float)(g.n * (int64_t)P), accumulate)));
         }
     }
     k_fixed_to_float<<<stream_blocks(g.n), kThreads, 0, s>>>(acc, g.n, maxbits, (float)(g.n * (int64_t)P), d_ref, accumulate);

@@ -690,3 +690,21 @@ def test_voxelize_backward_on_a_grid_of_2_31_rows():
     ref = oracle.voxelize_backward(patch, gs.mean, gs.scale, gs.quat, gs.value, d, 3.0)
     for x, r in zip(got, ref):
         assert rel_l2(host(x), np.asarray(r).reshape(tuple(x.shape))) <= 1e-4
+
+
+@pytest.mark.parametrize("n,P", [((16, 9, 5), 2), ((32, 17, 9), 2), ((97, 9, 5), 1), ((33, 33, 33), 13),
+                                 ((47, 33, 17), 21), ((32, 33, 33), 18)])
+def test_unfused_warp_tile_shapes(n, P):
+    """warp_volume and its adjoint on each tile: 32, 16 and 8 voxels wide (rows
+    that fill less of the wider ones), one plane per lane (few blocks) and two;
+    fp32 against the oracle within the bounds used above."""
+    grid = Grid(*n, 2.0, 2.0, 2.0)
+    rng = np.random.default_rng(460 + P)
+    V = rng.random(grid.shape).astype(np.float32)
+    D = (4.0 * rng.normal(size=(P, 3) + grid.shape)).astype(np.float32)
+    dW = rng.normal(size=(P,) + grid.shape).astype(np.float32)
+    assert rel_l2(host(pmf.warp_volume(grid, dev(V), dev(D))), oracle.warp(grid, V, D)) <= TOL32
+    dV, dD = pmf.warp_volume_backward(grid, dev(V), dev(D), dev(dW))
+    dV_ref, dD_ref = oracle.warp_backward(grid, V, D, dW)
+    assert rel_l2(host(dV), dV_ref) <= TOL32
+    assert rel_l2(host(dD), dD_ref) <= 1e-4
