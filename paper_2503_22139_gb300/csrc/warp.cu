@@ -1037,7 +1037,12 @@ __global__ void __launch_bounds__(kThreads) k_warp_bwd(GridD g, WarpTiles nt, co
 // read d_dvf twice and E per view and took 76 + 68 us at the paper grid (one
 // fp32 view), and a single thread per output summed the 608 partials in 53 us:
 // 54 us now, 336 MB being 50 us at the copy rate.  PG = 1 takes four voxels
-// per thread, PG = 4 two, what their sums leave registers for.
+// per thread, PG = 4 two, what their sums leave registers for (four bytes are
+// spilt at four levels, 52 at three: 130 us for four views at three levels, 474
+// in the two passes).  With one voxel per thread (an odd volume) the sums to
+// continue are read before the first is stored: read one by one, each behind the
+// store before it, nine views at four levels took 999 us, 867 in the two passes,
+// 455 now.  (Read ahead in runs too, one view at three levels takes 74 us, not 65.)
 template <typename T, int L, int PG, int V>
 __global__ void __launch_bounds__(kThreads, 2) k_combine_bwd(GridD g, int P, int p0, const T* __restrict__ E,
                                                           const float* __restrict__ w, const float* __restrict__ dD,
@@ -1060,6 +1065,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_combine_bwd(GridD g, int P, int
 #pragma unroll
                 for (int k = 0; k < 3; k++) ld_run<V>(dD + ((int64_t)(p0 + q) * 3 + k) * N + v, dd[q][k]);
             }
+        const bool more = accumulate || p0 > 0;
+        float ahead[V == 1 ? K : 1];  // one voxel per thread: the sums to continue
+        if (V == 1 && more) {
+#pragma unroll
+            for (int c = 0; c < K; c++) ahead[c] = dE[(int64_t)c * N + v];
+        }
 #pragma unroll
         for (int c = 0; c < K; c++) {  // c = 3 l + k
             float e[V], gE[V];
@@ -1067,11 +1078,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_combine_bwd(GridD g, int P, int
 #pragma unroll
             for (int i = 0; i < V; i++) gE[i] = 0.f;
             float* o = dE + (int64_t)c * N + v;
-            const bool more = accumulate || p0 > 0;
             float old[V];
             if (more) {
 #pragma unroll
-                for (int i = 0; i < V; i++) old[i] = o[i];
+                for (int i = 0; i < V; i++) old[i] = V == 1 ? ahead[V == 1 ? c : 0] : o[i];
                 if (p0 > 0) {
 #pragma unroll
                     for (int i = 0; i < V; i++) gE[i] = old[i];
