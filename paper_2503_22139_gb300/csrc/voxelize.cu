@@ -978,10 +978,11 @@ pmf_status gs_voxelize_tiled(const pmf_grid* grid, const pmf_gaussians* gs, pmf_
     GridD g = make_grid(grid);
     size_t fixed = vox_ws_layout(g, gs->n, 0, tl, nullptr, nullptr);
     if ((st = validate_ws(ws, ws_bytes, fixed)) != PMF_OK) return st;
-    // whatever is left after the fixed part holds the pair list
-    int64_t cap = (int64_t)((ws_bytes - fixed) / sizeof(unsigned)) + 1;
-    while (cap > 0 && vox_ws_layout(g, gs->n, cap, tl, nullptr, nullptr) > ws_bytes) cap -= 64;
-    if (cap < 0) cap = 0;
+    // whatever is left behind the fixed part, which ends in room for a list of one
+    // entry, holds the pair list: all of it, so that a list sized by the exact count
+    // lists every tile (entries short, the last tile scans all Gaussians: a
+    // 300,000-Gaussian call on 200 x 200 x 100 voxels took 1,321 us instead of 521)
+    int64_t cap = (int64_t)((ws_bytes - (fixed - align_up(sizeof(unsigned)))) / sizeof(unsigned));
     if (cap > 0xfffffff0ll) cap = 0xfffffff0ll;
     VoxWs w;
     vox_ws_layout(g, gs->n, cap, tl, &w, (char*)ws);

@@ -708,3 +708,19 @@ def test_unfused_warp_tile_shapes(n, P):
     dV_ref, dD_ref = oracle.warp_backward(grid, V, D, dW)
     assert rel_l2(host(dV), dV_ref) <= TOL32
     assert rel_l2(host(dD), dD_ref) <= 1e-4
+
+
+@pytest.mark.parametrize("tile", [None, (16, 8, 4)])
+@pytest.mark.parametrize("extra", [0, 1, 63])
+def test_voxelize_list_of_the_exact_count_lists_every_tile(tile, extra):
+    """A list with room for the counted pairs, whatever the count's place in the
+    workspace's 256-byte steps, holds them all: no tile scans every Gaussian (the
+    last one did), and the volume is the same."""
+    grid = Grid(30, 22, 13, 2.0, 2.0, 2.0)
+    pmf.device_counters(reset=True)
+    for n in (50, 57, 64, 71):
+        gs = gset(_rand_gaussians(470 + n, grid, n, 0.7, 3.0, 1), 3.0)
+        exact = pmf.gs_voxelize_count(grid, gs, tile)
+        got = pmf.gs_voxelize(grid, gs, pair_capacity=exact + extra, tile=tile)
+        assert torch.equal(got, pmf.gs_voxelize(grid, gs, tile=tile))
+    assert pmf.device_counters()["voxelize_list_overflow"] == 0
