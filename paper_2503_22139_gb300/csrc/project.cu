@@ -112,6 +112,107 @@ __device__ __forceinline__ void stage_plain(const T* __restrict__ V, const GridD
     }
 }
 
+// One sample from global memory, with the staged loops' position and blend.
+template <typename T>
+__device__ __forceinline__ float gather_one(const T* __restrict__ V, const GridD& g, const Ray& r, const int ib[3],
+                                            const float fb[3], float jf) {
+    const float ux = fmaf(jf, r.dh[0], fb[0]), uy = fmaf(jf, r.dh[1], fb[1]), uz = fmaf(jf, r.dh[2], fb[2]);
+    const float flx = floorf(ux), fly = floorf(uy), flz = floorf(uz);
+    return gather8(V, g, ib[0] + (int)flx, ib[1] + (int)fly, ib[2] + (int)flz, ux - flx, uy - fly, uz - flz);
+}
+
+// The eight corners of the interior cell whose lowest corner is element at (N < 2^31).
+template <typename T>
+__device__ __forceinline__ void load_cell(const T* __restrict__ V, int at, int sy, int sz, float v[8]) {
+#pragma unroll
+    for (int q = 0; q < 8; q++) v[q] = Store<T>::ld(V + at + ((q & 4) ? sz : 0) + ((q & 2) ? sy : 0), q & 1);
+}
+
+__device__ __forceinline__ bool interior(const int c[3], const GridD& g) {
+    return (unsigned)c[0] < (unsigned)(g.nx - 1) && (unsigned)c[1] < (unsigned)(g.ny - 1) &&
+           (unsigned)c[2] < (unsigned)(g.nz - 1);
+}
+
+// The samples [j0, j1] of one ray from global memory (the chunk's box is too
+// large to stage), added in sample order, so that every path (staged, bulk-copied
+// or gathered here) gives the same bits.  Latency bounds it, so interior samples
+// go in pairs, sixteen loads in flight: one by one, beside the unrolled staged
+// loop, 3 fp32 views of 201 x 199 x 99 voxels on a 96 x 70 detector took 768 us,
+// 600 so; 8 bf16 views of 200 x 200 x 100 at one-voxel steps, half the chunks
+// gathered, 1,047 and 935.  A pair that leaves the interior is taken one by one:
+// fp32 from the cells it has, the 16-bit types, whose conversions leave no
+// registers to keep them in, from the start (3 bf16 views of 200 x 200 x 100 on
+// the small detector 554 us, 610 with the cells kept).
+template <typename T>
+__device__ __forceinline__ void gather_global(const T* __restrict__ V, const GridD& g, const Ray& r, const int ib[3],
+                                              const float fb[3], int j0, int j1, float& acc) {
+    const int sy = g.nx, sz = g.nx * g.ny;
+    float jf = (float)j0;
+    if constexpr (sizeof(T) == 4) {
+        int j = j0;
+        for (; j + 1 <= j1; j += 2, jf += 2.0f) {
+            int c[2][3];
+            float f[2][3], v[2][8];
+            bool in = true;
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+#pragma unroll
+                for (int t = 0; t < 3; t++) {
+                    const float p = fmaf(jf + (float)u, r.dh[t], fb[t]), fl = floorf(p);
+                    c[u][t] = ib[t] + (int)fl;
+                    f[u][t] = p - fl;
+                }
+                in = in && interior(c[u], g);
+            }
+            if (in) {
+#pragma unroll
+                for (int u = 0; u < 2; u++) load_cell(V, (c[u][2] * g.ny + c[u][1]) * g.nx + c[u][0], sy, sz, v[u]);
+#pragma unroll
+                for (int u = 0; u < 2; u++) acc += trilin8(v[u], f[u][0], f[u][1], f[u][2]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 2; u++)
+                    acc += trilin_cell(V, g, c[u][0], c[u][1], c[u][2], f[u][0], f[u][1], f[u][2]);
+            }
+        }
+        for (; j <= j1; j++, jf += 1.0f) {  // the odd one
+            const float ux = fmaf(jf, r.dh[0], fb[0]), uy = fmaf(jf, r.dh[1], fb[1]), uz = fmaf(jf, r.dh[2], fb[2]);
+            const float flx = floorf(ux), fly = floorf(uy), flz = floorf(uz);
+            acc += trilin_cell(V, g, ib[0] + (int)flx, ib[1] + (int)fly, ib[2] + (int)flz, ux - flx, uy - fly, uz - flz);
+        }
+    } else {
+        const float jl = (float)j1;
+#pragma unroll 1
+        for (; jf < jl; jf += 2.0f) {
+            int at[2];
+            float f[2][3], v[2][8];
+            bool in = true;
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                int c[3];
+#pragma unroll
+                for (int t = 0; t < 3; t++) {
+                    const float p = fmaf(jf + (float)u, r.dh[t], fb[t]), fl = floorf(p);
+                    c[t] = ib[t] + (int)fl;
+                    f[u][t] = p - fl;
+                }
+                in = in && interior(c, g);
+                at[u] = (c[2] * g.ny + c[1]) * g.nx + c[0];
+            }
+            if (in) {
+#pragma unroll
+                for (int u = 0; u < 2; u++) load_cell(V, at[u], sy, sz, v[u]);
+                acc += trilin8(v[0], f[0][0], f[0][1], f[0][2]);
+                acc += trilin8(v[1], f[1][0], f[1][1], f[1][2]);
+            } else {
+                acc += gather_one(V, g, r, ib, fb, jf);
+                acc += gather_one(V, g, r, ib, fb, jf + 1.0f);
+            }
+        }
+        if (jf == jl) acc += gather_one(V, g, r, ib, fb, jf);
+    }
+}
+
 // One 16 x (RPB/16) pixel tile of view p: every thread of the CTA calls it.
 template <typename T, int CH, int RPB>
 __device__ __forceinline__ void project_tile(const GridD& g, int nu, int nv, int ntu, float step,
@@ -154,17 +255,7 @@ __device__ __forceinline__ void project_tile(const GridD& g, int nu, int nv, int
                 else gather_samples<65, kPlainBox, false>(r, box, q0, sz, j0, j1, fb, acc);
             }
         } else if (act) {
-            // the staged loop's own positions and blend, so that every path
-            // (staged, bulk-copied, or gathered from global memory) gives the
-            // same bits
-            float jf = (float)j0;
-            for (int j = j0; j <= j1; j++, jf += 1.0f) {
-                const float ux = fmaf(jf, r.dh[0], fb[0]), uy = fmaf(jf, r.dh[1], fb[1]),
-                            uz = fmaf(jf, r.dh[2], fb[2]);
-                const float flx = floorf(ux), fly = floorf(uy), flz = floorf(uz);
-                acc += gather8(V, g, ib[0] + (int)flx, ib[1] + (int)fly, ib[2] + (int)flz, ux - flx, uy - fly,
-                               uz - flz);
-            }
+            gather_global(V, g, r, ib, fb, j0, j1, acc);
         }
         __syncthreads();
     }

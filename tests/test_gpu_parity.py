@@ -724,3 +724,21 @@ def test_voxelize_list_of_the_exact_count_lists_every_tile(tile, extra):
         got = pmf.gs_voxelize(grid, gs, pair_capacity=exact + extra, tile=tile)
         assert torch.equal(got, pmf.gs_voxelize(grid, gs, tile=tile))
     assert pmf.device_counters()["voxelize_list_overflow"] == 0
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("n", [(41, 40, 39), (3, 2, 1)])
+def test_project_gathered_chunks(n, dt):
+    """Chunks whose box is too large to stage gather in pairs, from volumes with no
+    16-byte rows: interior pairs, pairs across the volume's faces (every pair of
+    the thin volume) and odd rests, against the oracle on the stored values."""
+    grid = Grid(*n, 0.5, 0.5, 0.5)
+    vw = circular_views(3, 60.0, 90.0, 18, 17, 12.0, 12.0, start=0.3)
+    det = Detector(18, 17, 0.25)
+    vol = dev(np.random.default_rng(490).random(grid.shape)).to(dt)
+    pmf.device_counters(reset=True)
+    got = pmf.conebeam_project(grid, det, views(vw), vol, shared=True)
+    if n[0] > 3:
+        assert pmf.device_counters(reset=True)["project_box_fallback"] > 0
+    ref = oracle.project(grid, 18, 17, 0.25, vw, host(vol))
+    assert rel_l2(host(got), ref) <= TOL32
