@@ -780,41 +780,65 @@ __global__ void __launch_bounds__(32 * kBwdItemWarps, (C == 1 ? 32 : 24) / kBwdI
     }
 }
 
-// The same for one slab per Gaussian and a grid with fewer voxels than a few per
-// Gaussian -- a crop, most of the set outside it: a warp takes eight Gaussians, each
-// lane finds one's voxel box, the empty ones' zero gradients are written by their
-// own lanes, and the warp walks the others one after the other.  (100,000
-// Gaussians, a 32^3 crop: a warp per Gaussian took 62 us, nearly all of it warps
-// that return at once; 28 us so.  On a whole volume the walk's
-// registers spill and cost a tenth, so that stays with a warp per Gaussian.)
-constexpr int kSparsePer = 8;
+// The same in two launches for many Gaussians on few voxels (bwd_listed): a crop,
+// most of the set outside it.  One lane per Gaussian writes the empty ones' zero
+// gradients and lists the others, then one-warp CTAs, as many as the GPU holds,
+// take the list's Gaussians one after the other, each the next that is left.
+// Launching a CTA costs about 0.6 ns however soon it returns: 100,000 Gaussians, a
+// 32^3 crop, 68 us with a warp each, 32 so.  The Gaussians' outputs are their own,
+// so the list's order, which is not fixed, does not show.
+struct BwdList {
+    unsigned count, next;  // Gaussians listed; tickets drawn beyond the CTAs' first
+};  // the list itself, [n], follows
 
 template <int C>
-__global__ void __launch_bounds__(32, C == 1 ? 32 : 24) k_vox_bwd_sparse(pmf_gaussians G, GridD g,
-                                                                         const float* __restrict__ dout, float* d_mean,
-                                                                         float* d_scale, float* d_quat, float* d_value,
-                                                                         int accumulate, bool vec) {
-    __shared__ WarpPlan plan;
+__global__ void __launch_bounds__(256) k_vox_bwd_list(pmf_gaussians G, GridD g, float* d_mean, float* d_scale,
+                                                      float* d_quat, float* d_value, int accumulate, BwdList* list) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
-    const int64_t first = (int64_t)blockIdx.x * kSparsePer, mine = first + lane;
     bool full = false;
-    if (lane < kSparsePer && mine < G.n) {
+    if (i < G.n) {
         GaussSetup st;
-        gauss_setup(G, mine, g, G.kappa, st);
+        gauss_setup(G, i, g, G.kappa, st);
         full = st.lo[0] <= st.hi[0] && st.lo[1] <= st.hi[1] && st.lo[2] <= st.hi[2];
         if (!full && !accumulate) {
-            for (int a = 0; a < 3; a++) d_mean[3 * mine + a] = d_scale[3 * mine + a] = 0.0f;
-            for (int a = 0; a < 4; a++) d_quat[4 * mine + a] = 0.0f;
-            for (int c = 0; c < C; c++) d_value[mine * C + c] = 0.0f;
+            for (int a = 0; a < 3; a++) d_mean[3 * i + a] = d_scale[3 * i + a] = 0.0f;
+            for (int a = 0; a < 4; a++) d_quat[4 * i + a] = 0.0f;
+            for (int c = 0; c < C; c++) d_value[i * C + c] = 0.0f;
         }
     }
-    for (unsigned todo = __ballot_sync(0xffffffffu, full); todo; todo &= todo - 1) {
-        const int64_t i = first + __ffs(todo) - 1;
+    const unsigned m = __ballot_sync(0xffffffffu, full);
+    unsigned at = 0u;
+    if (lane == 0 && m) at = atomicAdd(&list->count, (unsigned)__popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (full) reinterpret_cast<unsigned*>(list + 1)[at + __popc(m & ((1u << lane) - 1u))] = (unsigned)i;
+}
+
+template <int C>
+constexpr int bwd_resident() { return C == 1 ? 32 : 24; }  // one-warp CTAs an SM holds
+
+template <int C>
+__global__ void __launch_bounds__(32, bwd_resident<C>()) k_vox_bwd_listed(pmf_gaussians G, GridD g,
+                                                                           const float* __restrict__ dout,
+                                                                           float* d_mean, float* d_scale, float* d_quat,
+                                                                           float* d_value, int accumulate, bool vec,
+                                                                           BwdList* list) {
+    __shared__ WarpPlan plan;
+    __shared__ unsigned ticket;
+    const int lane = threadIdx.x & 31;
+    const unsigned count = list->count;
+    const unsigned* item = reinterpret_cast<const unsigned*>(list + 1);
+    for (unsigned k = blockIdx.x; k < count;) {
+        if (lane == 0) ticket = gridDim.x + atomicAdd(&list->next, 1u);  // drawn early: its latency is behind the work
+        const int64_t i = item[k];
         GaussSetup st;
         gauss_setup(G, i, g, G.kappa, st);
         float r[C + kMom];
         item_moments<C, false>(G, i, st, g, dout, 0, 1, vec, plan, r);
         if (lane == 0) moments_to_grad<C>(st, r, i, d_mean, d_scale, d_quat, d_value, accumulate);
+        __syncwarp();
+        k = ticket;
+        __syncwarp();  // read by all before the next one is drawn
     }
 }
 
@@ -849,6 +873,17 @@ int bwd_slabs(int64_t n) {
     int s = 1;
     while (s < 256 && n * s * 2 <= want) s *= 2;
     return s;
+}
+
+// Whether the adjoint lists the Gaussians that reach the grid: fewer than four
+// voxels per Gaussian (a whole volume at a usual density has more, a crop fewer)
+// and six of them for each resident CTA.  With every Gaussian inside it is no
+// slower either (43^3 voxels, one channel: 50,000 Gaussians 149 us, 143 with a warp
+// each; 150,000 382 and 391; three channels 184 and 186, 481 and 518), with nine
+// tenths outside 43 and 57, 72 and 119; at 20,000, all inside, it takes 79 us and a
+// warp each 70.
+bool bwd_listed(const GridD& g, int64_t n) {
+    return g.n < 4 * n && n >= 6 * 152 * 32 && (int64_t)g.ny * g.nz <= INT32_MAX;
 }
 
 pmf_status validate_gaussians(const pmf_gaussians* g) {
@@ -1019,6 +1054,7 @@ pmf_status gs_voxelize_backward_workspace(const pmf_grid* grid, int64_t n, int32
     if (channels > kMaxC) return set_error(PMF_EUNSUPPORTED, "channels > %d not supported", kMaxC);
     const int S = bwd_slabs(n);
     *bytes = S > 1 ? align_up(sizeof(float) * (size_t)n * S * (channels + kMom)) : 0;
+    if (S == 1 && bwd_listed(make_grid(grid), n)) *bytes = align_up(sizeof(BwdList) + sizeof(unsigned) * (size_t)n);
     return PMF_OK;
 }
 
@@ -1043,13 +1079,19 @@ pmf_status gs_voxelize_backward(const pmf_grid* grid, const pmf_gaussians* gs, c
     const unsigned nb = (unsigned)((items + kBwdItemWarps - 1) / kBwdItemWarps);
     const unsigned nf = (unsigned)((gs->n + kBwdWarps - 1) / kBwdWarps);
     const int T = 32 * kBwdWarps, TI = 32 * kBwdItemWarps;
-    const unsigned ns = (unsigned)((gs->n + kSparsePer - 1) / kSparsePer);
     const bool wide = (int64_t)g.ny * g.nz > INT32_MAX;
-    const bool sparse = S == 1 && g.n < 4 * gs->n && !wide;
+    const bool listed = S == 1 && bwd_listed(g, gs->n);
+    BwdList* list = (BwdList*)ws;
+    if (listed) cudaMemsetAsync(list, 0, sizeof(BwdList), s);
 #define PMF_VB(CC)                                                                                               \
-    if (sparse) k_vox_bwd_sparse<CC><<<ns, 32, 0, s>>>(*gs, g, d_out, d_mean, d_scale, d_quat, d_value, accumulate, vec); \
-    else if (wide) k_vox_bwd<CC, true><<<nb, TI, 0, s>>>(*gs, g, S, d_out, part, d_mean, d_scale, d_quat, d_value, accumulate, vec); \
-    else k_vox_bwd<CC, false><<<nb, TI, 0, s>>>(*gs, g, S, d_out, part, d_mean, d_scale, d_quat, d_value, accumulate, vec); \
+    if (listed) {                                                                                                \
+        k_vox_bwd_list<CC><<<(unsigned)((gs->n + 255) / 256), 256, 0, s>>>(*gs, g, d_mean, d_scale, d_quat, d_value, accumulate, list); \
+        k_vox_bwd_listed<CC><<<152 * bwd_resident<CC>(), 32, 0, s>>>(*gs, g, d_out, d_mean, d_scale, d_quat, d_value, accumulate, vec, list); \
+    } else if (wide) {                                                                                           \
+        k_vox_bwd<CC, true><<<nb, TI, 0, s>>>(*gs, g, S, d_out, part, d_mean, d_scale, d_quat, d_value, accumulate, vec); \
+    } else {                                                                                                     \
+        k_vox_bwd<CC, false><<<nb, TI, 0, s>>>(*gs, g, S, d_out, part, d_mean, d_scale, d_quat, d_value, accumulate, vec); \
+    }                                                                                                            \
     if (S > 1) k_vox_bwd_final<CC><<<nf, T, 0, s>>>(*gs, g, S, part, d_mean, d_scale, d_quat, d_value, accumulate);
     switch (gs->channels) {
         case 1: { PMF_VB(1) break; }

@@ -38,8 +38,8 @@ EQ14_DEFAULTS = dict(lambda_ssim=0.25, lambda_mbc=1.0, lambda_tv=0.05, tv_size=3
 
 def vox_bwd_launches(grid, gs) -> int:
     """Kernels one gs_voxelize_backward call launches: the slab pass, plus the
-    final pass when the set is split into several slabs (exactly when the call
-    needs a workspace)."""
+    final pass when the set is split into several slabs or the list pass when
+    the Gaussians in the grid are listed (exactly when the call needs a workspace)."""
     return 1 + (ops.gs_voxelize_backward_workspace(grid, gs.n, gs.channels) > 0)
 
 

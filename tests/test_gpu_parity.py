@@ -742,3 +742,39 @@ def test_project_gathered_chunks(n, dt):
         assert pmf.device_counters(reset=True)["project_box_fallback"] > 0
     ref = oracle.project(grid, 18, 17, 0.25, vw, host(vol))
     assert rel_l2(host(got), ref) <= TOL32
+
+
+@pytest.mark.parametrize("C,accumulate", [(1, False), (2, True), (3, False), (3, True), (4, False)])
+@pytest.mark.parametrize("n,G,listed", [((17, 16, 15), 29184, True), ((17, 16, 15), 30011, True),
+                                        ((17, 16, 15), 29183, False), ((53, 47, 41), 20011, False)])
+def test_voxelize_backward_listed_and_warp_each(n, G, listed, C, accumulate):
+    """The adjoint of a set too large to split: listed where there are fewer than
+    four voxels and enough Gaussians, else a warp each, also on a volume of more
+    voxels; about a third of the Gaussians outside get zero (or nothing added), a
+    sample of the others at every place of a warp, the last ones among them,
+    match the oracle within the bound used above."""
+    grid = Grid(*n, 2.0, 2.0, 2.0)
+    assert (4 * G > n[0] * n[1] * n[2]) == (n[0] < 50)
+    assert (pmf.ops.gs_voxelize_backward_workspace(grid, G, C) > 0) == listed
+    gs = _rand_gaussians(480, grid, G, 1.0, 4.0, C)
+    gs.mean[::3] += np.float32(400.0)  # outside
+    d = dev(np.random.default_rng(481).normal(size=(C,) + grid.shape))
+    base = tuple(torch.full((G, k), 0.25, device="cuda") for k in (3, 3, 4, C)) if accumulate else None
+    got = pmf.gs_voxelize_backward(grid, gset(gs, 3.0), d, grads=base, accumulate=accumulate)
+    zero = 0.25 if accumulate else 0.0
+    for x in got:
+        assert torch.all(x[::3] == zero)
+    sel = np.unique(np.concatenate([np.arange(0, G, 1499), np.arange(G - 8, G)]))
+    sel = sel[sel % 3 != 0]
+    ref = oracle.voxelize_backward(grid, gs.mean[sel], gs.scale[sel], gs.quat[sel], gs.value[sel], host(d), 3.0)
+    for x, r in zip(got, ref):
+        assert rel_l2(host(x)[sel] - zero, np.asarray(r).reshape(len(sel), -1)) <= 1e-4
+
+
+def test_voxelize_backward_list_of_none():
+    """A listed set with no Gaussian in the grid: zeros, or nothing added."""
+    grid, G = Grid(9, 8, 7, 2.0, 2.0, 2.0), 30000
+    gs = _rand_gaussians(482, grid, G, 1.0, 4.0, 1)
+    gs.mean[:] += np.float32(400.0)
+    d = torch.ones((1,) + grid.shape, device="cuda")
+    assert all(float(x.abs().max()) == 0.0 for x in pmf.gs_voxelize_backward(grid, gset(gs, 3.0), d))
