@@ -328,6 +328,15 @@ __device__ __forceinline__ bool block_reached(const float f[9], float k2, float 
     return !(t > 0.0f && t * t > fmaf(1.01f, k2, slack) * q);
 }
 
+// Whether a record's voxel box meets the tile at (x0, y0, z0).  A tile whose list
+// overflowed looks at every record, and most miss it: half a record decides
+// (2,000 Gaussians on 200 x 200 x 100 voxels, no list at all: 205 -> 165 us).
+__device__ __forceinline__ bool box_meets(const float4* rec, int x0, int y0, int z0, int tx, int ty, int tz) {
+    const float4 r2 = __ldg(rec + 2), r3 = __ldg(rec + 3);
+    return __float_as_int(r2.y) < x0 + tx && __float_as_int(r3.x) >= x0 && __float_as_int(r2.z) < y0 + ty &&
+           __float_as_int(r3.y) >= y0 && __float_as_int(r2.w) < z0 + tz && __float_as_int(r3.z) >= z0;
+}
+
 template <typename T, int C, int TX, int TY, int TZ>
 __global__ void __launch_bounds__(TX * TY * TZ / 2, 2048 / (TX * TY * TZ)) k_render(pmf_gaussians G, GridD g, VoxWs w, T* out, int ntx,
                                                              int nty) {
@@ -387,7 +396,7 @@ __global__ void __launch_bounds__(TX * TY * TZ / 2, 2048 / (TX * TY * TZ)) k_ren
         const int64_t k = base + tid;
         unsigned gi = 0u, occ = 0u;
         float f[9];
-        if (k < total) {
+        if (k < total && (listed || box_meets(w.rec + 4 * k, x0, y0, z0, TX, TY, TZ))) {
             gi = listed ? (PMF_DCHECK((long long)(off + k) < w.capacity) ? w.list[off + k] : 0u) : (unsigned)k;
             // the 4-voxel slices of the tile the voxel box reaches on each axis
             // (no voxel outside the box has q <= kappa^2), then the sub-blocks
