@@ -260,7 +260,7 @@ __device__ __forceinline__ void scatter_samples(const Ray& r, const Box& bx, int
 
 // One pixel tile of view p of the adjoint; box must be all zero on entry and is
 // all zero again on return.
-template <int CH, int RPB>
+template <int CH, int RPB, bool STAGED>
 __device__ __forceinline__ void backproject_tile(const GridD& g, int nu, int nv, int ntu, float step,
                                                  const pmf_view* __restrict__ views,
                                                  const float* __restrict__ dproj, int64_t vol_stride,
@@ -320,7 +320,7 @@ __device__ __forceinline__ void backproject_tile(const GridD& g, int nu, int nv,
         const Box bx = read_box(bs, sel);
         const int pitch = bx.bx <= 32 ? 33 : 65;
         const int sz = plane_stride(bx.by, pitch);
-        const bool fits = bx.vol > 0 && bx.bx <= 64 && (long long)bx.bz * sz <= box_words<CH>();
+        const bool fits = STAGED && bx.vol > 0 && bx.bx <= 64 && (long long)bx.bz * sz <= box_words<CH>();
         if (threadIdx.x == 0 && bx.vol > 0 && !fits) diag_count(PMF_DIAG_BACKPROJECT_BOX_FALLBACK);
         if (fits) {
             if (act) {
@@ -372,7 +372,7 @@ __device__ __forceinline__ void backproject_tile(const GridD& g, int nu, int nv,
     }
 }
 
-template <int CH, int RPB>
+template <int CH, int RPB, bool STAGED>
 __global__ void __launch_bounds__(RPB, 768 / RPB) k_backproject(GridD g, int nu, int nv, int ntu, float step,
                                                       const pmf_view* __restrict__ views,
                                                       const float* __restrict__ dproj, int64_t vol_stride,
@@ -382,8 +382,9 @@ __global__ void __launch_bounds__(RPB, 768 / RPB) k_backproject(GridD g, int nu,
     __shared__ BoxState bs;
     __shared__ unsigned sgmax;
     __shared__ float gsum[RPB / 32];
-    for (int i = threadIdx.x; i < box_words<CH>(); i += RPB) box[i] = 0;
-    backproject_tile<CH, RPB>(g, nu, nv, ntu, step, views, dproj, vol_stride, acc, maxbits, bound_mult, samples_per_voxel,
+    if (STAGED)  // without a box there is no dynamic shared memory
+        for (int i = threadIdx.x; i < box_words<CH>(); i += RPB) box[i] = 0;
+    backproject_tile<CH, RPB, STAGED>(g, nu, nv, ntu, step, views, dproj, vol_stride, acc, maxbits, bound_mult, samples_per_voxel,
                      blockIdx.y, blockIdx.x, box, bs, sgmax, gsum);
 }
 
@@ -447,17 +448,18 @@ __global__ void k_fixed_to_float_f4(const unsigned long long* __restrict__ acc, 
     if (MAX) block_max_bits(m, out_max);
 }
 
-template <int CH, int RPB>
+template <int CH, int RPB, bool STAGED>
 __global__ void __launch_bounds__(RPB, 768 / RPB) k_backproject_batched(const __grid_constant__ ProjBatch B) {
     extern __shared__ int box[];  // box_words<CH>()
     __shared__ BoxState bs;
     __shared__ unsigned sgmax;
     __shared__ float gsum[RPB / 32];
-    for (int i = threadIdx.x; i < box_words<CH>(); i += RPB) box[i] = 0;
+    if (STAGED)
+        for (int i = threadIdx.x; i < box_words<CH>(); i += RPB) box[i] = 0;
     for (int64_t w = blockIdx.x; w < B.total; w += gridDim.x) {
         const ProjItem it = B.it[find_item(B, w)];  // a copy: the tile code reads registers, not the parameter block
         const int local = (int)(w - it.begin);  // < 2^31: checked when the item is filled
-        backproject_tile<CH, RPB>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, it.dproj, it.vol_stride, it.acc, it.maxbits,
+        backproject_tile<CH, RPB, STAGED>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, it.dproj, it.vol_stride, it.acc, it.maxbits,
                          it.bound_mult, it.spv, local / it.ntiles, local % it.ntiles, box, bs, sgmax,
                          gsum);
         __syncthreads();
@@ -476,7 +478,7 @@ __global__ void __launch_bounds__(RPB, 768 / RPB) k_backproject_batched1(const _
     const int64_t w = blockIdx.x;
     const ProjItem it = B.it[find_item(B, w)];
     const int local = (int)(w - it.begin);
-    backproject_tile<CH, RPB>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, it.dproj, it.vol_stride, it.acc, it.maxbits,
+    backproject_tile<CH, RPB, true>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, it.dproj, it.vol_stride, it.acc, it.maxbits,
                      it.bound_mult, it.spv, local / it.ntiles, local % it.ntiles, box, bs, sgmax, gsum);
 }
 
@@ -506,6 +508,13 @@ __global__ void k_fixed_to_float_batched(const __grid_constant__ ProjBatch B, in
     if (MAX) block_max_bits(m, out_max);
 }
 
+// Whether the scatter's cells are exact (kFloorBias: positions below 2^22; the index
+// of the cell is formed from integers).
+bool box_exact(const pmf_grid& g, float step, int chunk) { return cells_exact(g, step, chunk, 1.0, 1.0, 4194304.0); }
+
+// The chunk and rays of the kernels without a box.
+constexpr int kFarChunk = 48, kFarRays = 128;
+
 pmf_status backproject_grid(const pmf_grid* grid, const pmf_detector* det, int32_t P, const pmf_view* views,
                             const float* d_proj, float* d_vol, int64_t vol_stride, int accumulate, void* ws,
                             size_t ws_bytes, const MarchShape& sh, cudaStream_t s, unsigned* out_max = nullptr) {
@@ -528,13 +537,17 @@ pmf_status backproject_grid(const pmf_grid* grid, const pmf_detector* det, int32
         const int64_t nq = Q * P;
         int64_t nb = (nq + 255) / 256;
         k_absmax_f<<<(unsigned)(nb < 1024 ? nb : 1024), 256, 0, s>>>(d_proj, nq, maxbits);
-        const int ntu = (det->nu + 15) / 16, ntv = tiles_v(det->nv, sh.rays);
+        const bool staged = box_exact(*grid, det->step_mm, sh.chunk);
+        const int ntu = (det->nu + 15) / 16, ntv = tiles_v(det->nv, staged ? sh.rays : kFarRays);
         dim3 gr((unsigned)(ntu * ntv), (unsigned)P);
-        const float spv = chunk_samples_per_voxel(grid, det->step_mm, sh.chunk);
-        PMF_DISPATCH_ADJOINT(sh, CH, RPB, {
+        const float spv = chunk_samples_per_voxel(grid, det->step_mm, staged ? sh.chunk : kFarChunk);
+        if (!staged)
+            k_backproject<kFarChunk, kFarRays, false><<<gr, kFarRays, 0, s>>>(g, det->nu, det->nv, ntu, det->step_mm, views, d_proj,
+                                                                             vol_stride, acc, maxbits, bound_mult, spv);
+        else PMF_DISPATCH_ADJOINT(sh, CH, RPB, {
             constexpr int smem = (int)sizeof(int) * box_words<CH>();
-            cudaFuncSetAttribute(k_backproject<CH, RPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            k_backproject<CH, RPB><<<gr, RPB, smem, s>>>(g, det->nu, det->nv, ntu, det->step_mm, views, d_proj, vol_stride, acc,
+            cudaFuncSetAttribute(k_backproject<CH, RPB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            k_backproject<CH, RPB, true><<<gr, RPB, smem, s>>>(g, det->nu, det->nv, ntu, det->step_mm, views, d_proj, vol_stride, acc,
                                                       maxbits, bound_mult, spv);
         });
     }
@@ -570,16 +583,19 @@ pmf_status backproject_batched_impl(int32_t n, const pmf_backproject_item* items
     char* cur = (char*)ws;
     int ord[kMaxItems];
     longest_first(n, items, ord);  // work-list position k holds item ord[k]
+    bool staged = true;
+    for (int k = 0; k < n; k++) staged = staged && box_exact(items[k].grid, items[k].det.step_mm, sh.chunk);
+    const int rays = staged ? sh.rays : kFarRays;
     for (int k = 0; k < n; k++) {
         const pmf_backproject_item& in = items[ord[k]];
         pmf_project_item tmp{in.grid, in.det, in.P, in.views, nullptr, in.vol_stride, nullptr};
-        if ((st = fill_item(tmp, total, sh.rays, B.it[k])) != PMF_OK) return st;
+        if ((st = fill_item(tmp, total, rays, B.it[k])) != PMF_OK) return st;
         PMF_REQUIRE(in.d_vol != nullptr && (in.P == 0 || in.d_proj != nullptr), "item %d: null pointer", ord[k]);
         ProjItem& it = B.it[k];
         const int64_t Q = (int64_t)in.det.nu * in.det.nv;
         const double rays = (double)Q * (in.vol_stride ? 1.0 : (double)in.P);
         it.bound_mult = (float)((double)in.det.step_mm * rays * (double)max_samples_per_voxel(&in.grid, in.det.step_mm));
-        it.spv = chunk_samples_per_voxel(&in.grid, in.det.step_mm, sh.chunk);
+        it.spv = chunk_samples_per_voxel(&in.grid, in.det.step_mm, staged ? sh.chunk : kFarChunk);
         it.dproj = in.d_proj;
         it.dvol = in.d_vol;
         it.maxbits = (unsigned*)cur;
@@ -601,15 +617,16 @@ pmf_status backproject_batched_impl(int32_t n, const pmf_backproject_item* items
     if (total > 0) {
         int ntl[kMaxItems];
         for (int i = 0; i < n; i++) ntl[i] = B.it[i].ntiles;
-        const unsigned nc = persistent_ctas(total, ctas, sh.rays, ntl, n);
-        PMF_DISPATCH_ADJOINT(sh, CH, RPB, {
+        const unsigned nc = persistent_ctas(total, ctas, rays, ntl, n);
+        if (!staged) k_backproject_batched<kFarChunk, kFarRays, false><<<nc, kFarRays, 0, s>>>(B);
+        else PMF_DISPATCH_ADJOINT(sh, CH, RPB, {
             constexpr int smem = (int)sizeof(int) * box_words<CH>();
             if ((int64_t)nc == total) {
                 cudaFuncSetAttribute(k_backproject_batched1<CH, RPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
                 k_backproject_batched1<CH, RPB><<<nc, RPB, smem, s>>>(B);
             } else {
-                cudaFuncSetAttribute(k_backproject_batched<CH, RPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                k_backproject_batched<CH, RPB><<<nc, RPB, smem, s>>>(B);
+                cudaFuncSetAttribute(k_backproject_batched<CH, RPB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                k_backproject_batched<CH, RPB, true><<<nc, RPB, smem, s>>>(B);
             }
         });
     }

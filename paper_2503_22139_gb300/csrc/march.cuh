@@ -363,6 +363,18 @@ float chunk_samples_per_voxel(const pmf_grid* grid, float step, int chunk) {
     return (float)fmin(s, (double)chunk);
 }
 
+// Whether the staged loops find every cell of a box that fits.  They index it with
+// floats: a sample's cell relative to its ray's anchor, which on each axis is within
+// `chunk` steps and two cells of zero, times the words (1, wy, wz) a cell is apart,
+// exact below `limit`.  False also for steps that are infinite in voxels (a NaN
+// position has no cell).  Such calls take the kernels without staging, whose cells
+// are checked integers.
+bool cells_exact(const pmf_grid& g, float step, int chunk, double wy, double wz, double limit) {
+    const double reach = (double)chunk * (double)step;
+    return reach < 3.0e38 * fmin(fmin((double)g.vx, (double)g.vy), (double)g.vz) &&
+           reach * (1.0 / g.vx + wy / g.vy + wz / g.vz) + 2.0 * (1.0 + wy + wz) < limit;
+}
+
 int max_samples_per_voxel(const pmf_grid* grid, float step) {
     // a ray crosses the open 2x2x2-voxel support of one voxel over at most its
     // diagonal, 2 |v|, so it takes at most floor(2|v| / step) + 1 samples there

@@ -213,8 +213,9 @@ __device__ __forceinline__ void gather_global(const T* __restrict__ V, const Gri
     }
 }
 
-// One 16 x (RPB/16) pixel tile of view p: every thread of the CTA calls it.
-template <typename T, int CH, int RPB>
+// One 16 x (RPB/16) pixel tile of view p: every thread of the CTA calls it.  Not
+// STAGED: every chunk is gathered (plain_exact).
+template <typename T, int CH, int RPB, bool STAGED>
 __device__ __forceinline__ void project_tile(const GridD& g, int nu, int nv, int ntu, float step,
                                              const pmf_view* __restrict__ views, const T* __restrict__ vol,
                                              int64_t vol_stride, float* __restrict__ proj, int p, int tile,
@@ -243,7 +244,7 @@ __device__ __forceinline__ void project_tile(const GridD& g, int nu, int nv, int
         const Box bx = read_box(bs, sel);
         int sz;
         const int pitch = bx.vol > 0 ? plain_layout(bx, sz) : 0;
-        const bool fits = pitch > 0;
+        const bool fits = STAGED && pitch > 0;
         if (threadIdx.x == 0 && bx.vol > 0 && !fits) diag_count(PMF_DIAG_PROJECT_BOX_FALLBACK);
         if (fits) {
             stage_plain<T, RPB>(V, g, bx, pitch, sz, box);
@@ -262,13 +263,13 @@ __device__ __forceinline__ void project_tile(const GridD& g, int nu, int nv, int
     if (in) proj[((int64_t)p * nv + b) * nu + a] = step * acc;
 }
 
-template <typename T, int CH, int RPB>
+template <typename T, int CH, int RPB, bool STAGED>
 __global__ void __launch_bounds__(RPB, 1024 / RPB) k_project(GridD g, int nu, int nv, int ntu, float step,
                                                   const pmf_view* __restrict__ views, const T* __restrict__ vol,
                                                   int64_t vol_stride, float* __restrict__ proj) {
     extern __shared__ __align__(128) float box[];  // kPlainBox floats
     __shared__ BoxState bs;
-    project_tile<T, CH, RPB>(g, nu, nv, ntu, step, views, vol, vol_stride, proj, blockIdx.y, blockIdx.x, box, bs);
+    project_tile<T, CH, RPB, STAGED>(g, nu, nv, ntu, step, views, vol, vol_stride, proj, blockIdx.y, blockIdx.x, box, bs);
 }
 
 // ------------------------------------------- forward with bulk-copy staging
@@ -491,14 +492,14 @@ __global__ void __launch_bounds__(RPB, 1024 / RPB) k_project_batched_tma(const _
     }
 }
 
-template <typename T, int CH, int RPB>
+template <typename T, int CH, int RPB, bool STAGED>
 __global__ void __launch_bounds__(RPB, 1024 / RPB) k_project_batched(const __grid_constant__ ProjBatch B) {
     extern __shared__ __align__(128) float box[];  // kPlainBox floats
     __shared__ BoxState bs;
     for (int64_t w = blockIdx.x; w < B.total; w += gridDim.x) {
         const ProjItem it = B.it[find_item(B, w)];  // a copy: the tile code reads registers, not the parameter block
         const int local = (int)(w - it.begin);  // < 2^31: checked when the item is filled
-        project_tile<T, CH, RPB>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, (const T*)it.vol, it.vol_stride, it.proj,
+        project_tile<T, CH, RPB, STAGED>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, (const T*)it.vol, it.vol_stride, it.proj,
                         local / it.ntiles, local % it.ntiles, box, bs);
         __syncthreads();
     }
@@ -532,7 +533,7 @@ __global__ void __launch_bounds__(RPB, 1024 / RPB) k_project_batched1(const __gr
     const int64_t w = blockIdx.x;
     const ProjItem it = B.it[find_item(B, w)];
     const int local = (int)(w - it.begin);
-    project_tile<T, CH, RPB>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, (const T*)it.vol, it.vol_stride, it.proj,
+    project_tile<T, CH, RPB, true>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, (const T*)it.vol, it.vol_stride, it.proj,
                     local / it.ntiles, local % it.ntiles, box, bs);
 }
 
@@ -551,6 +552,21 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     }();
     return fn;
 }
+
+// Whether the plain kernel's cell index is exact (integers of floats below 2^24): up
+// to steps of about 50 of the smallest voxels.  A box that fits has planes of at
+// most half its words and rows of at most 65.
+bool plain_exact(const pmf_grid& g, float step, int chunk) {
+    return cells_exact(g, step, chunk, 65.0, 0.5 * kPlainBox, 16777216.0);
+}
+
+// The bulk-copy kernel's (kFloorBias: a quarter of that).
+bool bulk_exact(const pmf_grid& g, float step, int chunk) {
+    return cells_exact(g, step, chunk, kTmaX, 0.5 * kTmaBox, 4194304.0);
+}
+
+// The chunk and rays of the kernels without staging.
+constexpr int kFarChunk = 48, kFarRays = 256;
 
 // A 4-D map (x, y, z, volume) over fp32 volumes for the staged forward, or
 // false when the layout does not allow bulk copies (base or a stride not a
@@ -593,10 +609,18 @@ pmf_status project_grid(const pmf_grid* grid, const pmf_detector* det, int32_t P
     PMF_REQUIRE(vol && proj, "null pointer");
     PMF_REQUIRE(vol_stride >= 0, "vol_stride must be >= 0");
     GridD g = make_grid(grid);
-    const int ntu = (det->nu + 15) / 16, ntv = tiles_v(det->nv, sh.rays);
+    const int ntu = (det->nu + 15) / 16;
+    if (!plain_exact(*grid, det->step_mm, sh.chunk)) {
+        const dim3 gf((unsigned)(ntu * tiles_v(det->nv, kFarRays)), (unsigned)P);
+        PMF_DISPATCH_DTYPE(dtype, T, k_project<T, kFarChunk, kFarRays, false><<<gf, kFarRays, 0, s>>>(
+            g, det->nu, det->nv, ntu, det->step_mm, views, (const T*)vol, vol_stride, proj));
+        return check_launch("conebeam_project");
+    }
+    const int ntv = tiles_v(det->nv, sh.rays);
     dim3 gr((unsigned)(ntu * ntv), (unsigned)P);
     CUtensorMap map;
-    if (sh.tma && dtype == PMF_F32 && encode_volume_map(&map, (const float*)vol, grid, P, vol_stride)) {
+    if (sh.tma && dtype == PMF_F32 && bulk_exact(*grid, det->step_mm, sh.chunk) &&
+        encode_volume_map(&map, (const float*)vol, grid, P, vol_stride)) {
         PMF_DISPATCH_PROJ(sh, CH, RPB, {
             cudaFuncSetAttribute(k_project_tma<CH, RPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kTmaBox * sizeof(float)));
             k_project_tma<CH, RPB><<<gr, RPB, kTmaBox * sizeof(float), s>>>(g, det->nu, det->nv, ntu, det->step_mm, views, map,
@@ -605,8 +629,8 @@ pmf_status project_grid(const pmf_grid* grid, const pmf_detector* det, int32_t P
         return check_launch("conebeam_project");
     }
     PMF_DISPATCH_PROJ(sh, CH, RPB, PMF_DISPATCH_DTYPE(dtype, T, {
-        cudaFuncSetAttribute(k_project<T, CH, RPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kPlainBox * sizeof(float)));
-        k_project<T, CH, RPB><<<gr, RPB, kPlainBox * sizeof(float), s>>>(g, det->nu, det->nv, ntu, det->step_mm, views,
+        cudaFuncSetAttribute(k_project<T, CH, RPB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kPlainBox * sizeof(float)));
+        k_project<T, CH, RPB, true><<<gr, RPB, kPlainBox * sizeof(float), s>>>(g, det->nu, det->nv, ntu, det->step_mm, views,
                                                                         (const T*)vol, vol_stride, proj);
     }));
     return check_launch("conebeam_project");
@@ -623,9 +647,15 @@ pmf_status project_batched_impl(int32_t n, const pmf_project_item* items, pmf_dt
     int64_t total = 0;
     int ord[kMaxItems];
     longest_first(n, items, ord);  // work-list position k holds item ord[k]
+    bool staged = true, bulk = true;
+    for (int k = 0; k < n; k++) {
+        staged = staged && plain_exact(items[k].grid, items[k].det.step_mm, sh.chunk);
+        bulk = bulk && bulk_exact(items[k].grid, items[k].det.step_mm, sh.chunk);
+    }
+    const int rays = staged ? sh.rays : kFarRays;
     for (int k = 0; k < n; k++) {
         const pmf_project_item& in = items[ord[k]];
-        if ((st = fill_item(in, total, sh.rays, B.it[k])) != PMF_OK) return st;
+        if ((st = fill_item(in, total, rays, B.it[k])) != PMF_OK) return st;
         PMF_REQUIRE(in.P == 0 || (in.vol && in.proj), "item %d: null pointer", ord[k]);
         B.it[k].vol = in.vol;
         B.it[k].proj = in.proj;
@@ -635,8 +665,12 @@ pmf_status project_batched_impl(int32_t n, const pmf_project_item* items, pmf_dt
     if (total == 0) return PMF_OK;
     int ntl[kMaxItems];
     for (int i = 0; i < n; i++) ntl[i] = B.it[i].ntiles;
-    const unsigned nc = persistent_ctas(total, ctas, sh.rays, ntl, n);
-    if (sh.tma && dtype == PMF_F32) {
+    const unsigned nc = persistent_ctas(total, ctas, rays, ntl, n);
+    if (!staged) {
+        PMF_DISPATCH_DTYPE(dtype, T, k_project_batched<T, kFarChunk, kFarRays, false><<<nc, kFarRays, 0, s>>>(B));
+        return check_launch("conebeam_project_batched");
+    }
+    if (sh.tma && dtype == PMF_F32 && bulk) {
         ProjBatchTma tb{};
         bool all = true;
         for (int k = 0; k < n && all; k++) {
@@ -665,9 +699,9 @@ pmf_status project_batched_impl(int32_t n, const pmf_project_item* items, pmf_dt
                                  (int)(kPlainBox * sizeof(float)));
             k_project_batched1<T, CH, RPB><<<nc, RPB, kPlainBox * sizeof(float), s>>>(B);
         } else {
-            cudaFuncSetAttribute(k_project_batched<T, CH, RPB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(k_project_batched<T, CH, RPB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(kPlainBox * sizeof(float)));
-            k_project_batched<T, CH, RPB><<<nc, RPB, kPlainBox * sizeof(float), s>>>(B);
+            k_project_batched<T, CH, RPB, true><<<nc, RPB, kPlainBox * sizeof(float), s>>>(B);
         }
     }));
     return check_launch("conebeam_project_batched");

@@ -778,3 +778,38 @@ def test_voxelize_backward_list_of_none():
     gs.mean[:] += np.float32(400.0)
     d = torch.ones((1,) + grid.shape, device="cuda")
     assert all(float(x.abs().max()) == 0.0 for x in pmf.gs_voxelize_backward(grid, gset(gs, 3.0), d))
+
+
+@pytest.mark.parametrize("n", [(8, 8, 8), (9, 8, 7)])
+def test_marchers_take_steps_beyond_their_float_cells(n):
+    """Steps that are infinite in voxels along x (a voxel of 1.2e-38 mm) or tens of
+    thousands of voxels long leave the staged loops' float cells, so every such
+    chunk goes through global memory, whose cells are checked integers: the calls
+    return, the projections of the rays that cross are the NaN of a NaN position
+    (or the oracle's value), and the next call is the usual one's."""
+    vol = np.random.default_rng(491).random((2,) + n[::-1]).astype(np.float32)
+    dY = torch.ones((2, 16, 16), device="cuda")
+    vw = np.array([[0, -100, 1, 0, 100, 2, 1, 0, 0, 0, 0, 1.0], [3, -90, 0, -2, 110, 0, 1, 0, 0, 0, 0, 1.0]])
+    thin, det = Grid(*n, 1.2e-38, 10.0, 10.0), Detector(16, 16, 5.0)
+    pmf.device_counters(reset=True)
+    for dt in (torch.float32, torch.bfloat16):
+        Y = pmf.conebeam_project(thin, det, views(vw), dev(vol).to(dt))
+        assert torch.all(torch.isnan(Y) | (Y == 0)) and torch.isnan(Y).any()
+        Yb = pmf.conebeam_project_batched([(thin, det, views(vw), dev(vol).to(dt), False)])[0]
+        assert torch.equal(torch.isnan(Yb), torch.isnan(Y))
+    pmf.conebeam_project_backward(thin, det, views(vw), dY)
+    c = pmf.device_counters(reset=True)
+    assert c["project_box_fallback"] > 0 and c["backproject_box_fallback"] > 0 and c["timeout"] == 0
+    # a step of 60,000 voxels from a source inside the volume: sample 0 and none other
+    grid, far = Grid(*n, 2.0, 2.0, 2.0), Detector(16, 16, 120000.0)
+    inside = circular_views(2, 1.0, 60.0, 16, 16, 3.0, 3.0, start=0.2)
+    got = pmf.conebeam_project(grid, far, views(inside), dev(vol))
+    ref = oracle.project(grid, 16, 16, 120000.0, inside, vol)
+    assert rel_l2(host(got), ref) <= TOL32
+    gb = pmf.conebeam_project_backward(grid, far, views(inside), dY)
+    assert rel_l2(host(gb), oracle.project_backward(grid, 16, 16, 120000.0, inside, host(dY))) <= TOL32
+    near = Detector(16, 16, 1.0)
+    bt = pmf.conebeam_project_backward_batched([(grid, d, views(inside), dY, False) for d in (far, near)])
+    assert torch.equal(bt[0], gb)
+    refb = oracle.project_backward(grid, 16, 16, 1.0, inside, host(dY))
+    assert rel_l2(host(bt[1]), refb) <= TOL32
