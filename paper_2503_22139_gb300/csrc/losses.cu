@@ -16,9 +16,9 @@
 // in shared memory and evaluates SSIM and its partial derivatives per pixel.
 // Shared-memory loads bound both passes, so each thread forms four outputs
 // from one set of loads: four neighbours along x from 16-byte loads, four along
-// y from one column of 14 rows (41 loaded words a pixel; one output per thread
-// on 32x8 tiles took 105).  Eight 512 x 384 projections: forward 50 -> 35 us,
-// adjoint 31 -> 29 us.
+// y from one column of 14 rows (the forward loads 31 words a pixel; one output
+// per thread on 32x8 tiles loads 105).  Eight 512 x 384 projections: forward 50
+// -> 35 us, adjoint 31 -> 29 us.  Few pixels take the latter form (ssim_small).
 // The moments are taken about a per-tile shift (the tile's mean) so that
 // s^2 = E[x^2] - mu^2 does not cancel in fp32 at projection magnitudes; zero
 // padding is honoured exactly through the window mass s inside the image.
@@ -28,13 +28,17 @@
 namespace pmf {
 namespace {
 
-constexpr int kTU = 32, kTV = 16;                 // SSIM output tile
+constexpr int kTU = 32;                           // SSIM output tile's width
 constexpr int kHW = 5;                            // window half-width
-constexpr int kInU = kTU + 2 * kHW, kInV = kTV + 2 * kHW;
+constexpr int kInU = kTU + 2 * kHW;
 constexpr int kInP = 44;                          // row pitch of the staged tile: 16-byte rows
-constexpr int kRun = 4;                           // outputs per thread of either pass
-constexpr int kSsimThreads = kTU * kTV / kRun;    // 128
-static_assert(kInP % 4 == 0 && kInP >= kTU - kRun + 16 && kTU % kRun == 0 && kTV % kRun == 0, "runs of four");
+
+// RUN outputs per thread of either pass: 4 on tiles 16 high, 1 on tiles 8 high.
+template <int RUN>
+struct Ssim {
+    static constexpr int TV = RUN == 4 ? 16 : 8, IN_V = TV + 2 * kHW, THREADS = kTU * TV / RUN;
+    static_assert((RUN == 4 || RUN == 1) && kInP % 4 == 0 && kInP >= kTU - RUN + (RUN == 4 ? 16 : 11) && TV % RUN == 0, "runs");
+};
 
 // The normalised 1-D Gaussian window (sigma 1.5, 11 taps): w[t] for offset t - 5.
 struct Window {
@@ -75,39 +79,62 @@ __device__ __forceinline__ float block_sum_f(float v, float* red) {
     return t;
 }
 
-// The 16 staged words from column c of a row (c a multiple of 4).
-__device__ __forceinline__ void load16(const float* row, float v[16]) {
+// The staged words of RUN outputs from column c of a row (RUN 4: c a multiple of 4).
+template <int RUN>
+__device__ __forceinline__ void load_staged(const float* row, float v[16]) {
+    if constexpr (RUN == 4) {
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-        const float4 q = reinterpret_cast<const float4*>(row)[k];
-        v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
+        for (int k = 0; k < 4; k++) {
+            const float4 q = reinterpret_cast<const float4*>(row)[k];
+            v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 11; k++) v[k] = row[k];
     }
 }
 
-// f(row, column) once per staged word (kInV x kInP), a warp per row; unrolled,
-// so that a thread's loads overlap.
-template <class F>
+template <int RUN>
+__device__ __forceinline__ void store_run(float* p, const float v[RUN]) {
+    if constexpr (RUN == 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else p[0] = v[0];
+}
+
+// f(row, column) once per staged word, unrolled, so that a thread's loads overlap.
+// RUN 4: a warp per row, kInP columns.  RUN 1: the kInU columns that are read, all
+// threads busy.
+template <int RUN, class F>
 __device__ __forceinline__ void for_staged(const F& f) {
-    constexpr int W = kSsimThreads / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int NT = Ssim<RUN>::THREADS, W = NT / 32, kInV = Ssim<RUN>::IN_V;
+    if constexpr (RUN == 1) {
 #pragma unroll
-    for (int k = 0; k < (kInV + W - 1) / W; k++) {
-        const int r = warp + W * k;
-        if (r >= kInV) break;
-        f(r, lane);
-        if (lane + 32 < kInP) f(r, lane + 32);
+        for (int k = 0; k < (kInU * kInV + NT - 1) / NT; k++) {
+            const int i = threadIdx.x + NT * k;
+            if (i < kInU * kInV) f(i / kInU, i % kInU);
+        }
+    } else {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+        for (int k = 0; k < (kInV + W - 1) / W; k++) {
+            const int r = warp + W * k;
+            if (r >= kInV) break;
+            f(r, lane);
+            if (lane + 32 < kInP) f(r, lane + 32);
+        }
     }
 }
 
 // Forward: per pixel S and the partials G1 = dS/dmu_x - 2 mu_x G2 - mu_y G3,
 // G2 = dS/d s_x^2, G3 = dS/d s_xy (with dS/dmu_x taken at fixed s's), so that
 // dS(q)/dx(r) = w(q - r) (G1(q) + 2 x(r) G2(q) + y(r) G3(q)).
-__global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int ntu, const float* __restrict__ X,
+template <int RUN>
+__global__ void __launch_bounds__(Ssim<RUN>::THREADS) k_dssim_fwd(int nu, int nv, int ntu, const float* __restrict__ X,
                                                            const float* __restrict__ Y, float C1, float C2,
                                                            const Window W, float* G, double* part) {
+    constexpr int kTV = Ssim<RUN>::TV, kInV = Ssim<RUN>::IN_V, NT = Ssim<RUN>::THREADS;
     __shared__ __align__(16) float sx[kInV][kInP], sy[kInV][kInP];
     __shared__ __align__(16) float h[5][kInV][kTU];
-    __shared__ float red[2][kSsimThreads / 32];
+    __shared__ float red[2][NT / 32];
     const int p = blockIdx.y, tu = blockIdx.x % ntu, tv = blockIdx.x / ntu;
     const int u0 = tu * kTU - kHW, v0 = tv * kTV - kHW;
     const int64_t Q = (int64_t)nu * nv;
@@ -115,7 +142,7 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int 
     const float* Yp = Y + (int64_t)p * Q;
     // stage the tile and halo (zero outside the image) and its mean over the image part
     float ax = 0.f, ay = 0.f;
-    for_staged([&](int r, int c) {
+    for_staged<RUN>([&](int r, int c) {
         const int u = u0 + c, v = v0 + r;
         const bool in = c < kInU && u >= 0 && u < nu && v >= 0 && v < nv;
         const float x = in ? __ldg(Xp + (int64_t)v * nu + u) : 0.f, y = in ? __ldg(Yp + (int64_t)v * nu + u) : 0.f;
@@ -135,13 +162,13 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int 
     __syncthreads();
     const float n_in = (float)((min(u0 + kInU, nu) - max(u0, 0)) * (min(v0 + kInV, nv) - max(v0, 0)));
     ax = ay = 0.f;
-    for (int k = 0; k < kSsimThreads / 32; k++) {  // fixed order, same in every thread
+    for (int k = 0; k < NT / 32; k++) {  // fixed order, same in every thread
         ax += red[0][k];
         ay += red[1][k];
     }
     const float cx = ax / n_in, cy = ay / n_in;
     // shift inside the image (outside stays zero)
-    for_staged([&](int r, int c) {
+    for_staged<RUN>([&](int r, int c) {
         const int u = u0 + c, v = v0 + r;
         if (c < kInU && u >= 0 && u < nu && v >= 0 && v < nv) {
             sx[r][c] -= cx;
@@ -150,20 +177,20 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int 
     });
     __syncthreads();
     // horizontal pass: 5 sums for every staged row and output column, four columns per thread
-    for (int i = threadIdx.x; i < kInV * (kTU / kRun); i += kSsimThreads) {
-        const int r = i / (kTU / kRun), c = (i - r * (kTU / kRun)) * kRun;
-        float x[16], y[16], m[5][kRun];
-        load16(&sx[r][c], x);
-        load16(&sy[r][c], y);
+    for (int i = threadIdx.x; i < kInV * (kTU / RUN); i += NT) {
+        const int r = i / (kTU / RUN), c = (i - r * (kTU / RUN)) * RUN;
+        float x[16], y[16], m[5][RUN];
+        load_staged<RUN>(&sx[r][c], x);
+        load_staged<RUN>(&sy[r][c], y);
 #pragma unroll
         for (int k = 0; k < 5; k++)
 #pragma unroll
-            for (int o = 0; o < kRun; o++) m[k][o] = 0.f;
+            for (int o = 0; o < RUN; o++) m[k][o] = 0.f;
 #pragma unroll
-        for (int e = 0; e < 10 + kRun; e++) {
+        for (int e = 0; e < 10 + RUN; e++) {
             const float xx = x[e] * x[e], yy = y[e] * y[e], xy = x[e] * y[e];
 #pragma unroll
-            for (int o = 0; o < kRun; o++) {
+            for (int o = 0; o < RUN; o++) {
                 const int t = e - o;
                 if (t < 0 || t > 10) continue;
                 m[0][o] = fmaf(W.w[t], x[e], m[0][o]);
@@ -175,24 +202,24 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int 
         }
 #pragma unroll
         for (int k = 0; k < 5; k++)
-            *reinterpret_cast<float4*>(&h[k][r][c]) = make_float4(m[k][0], m[k][1], m[k][2], m[k][3]);
+            store_run<RUN>(&h[k][r][c], m[k]);
     }
     __syncthreads();
     // vertical pass: four output rows of one column per thread
-    const int c = threadIdx.x % kTU, r0 = threadIdx.x / kTU * kRun;
+    const int c = threadIdx.x % kTU, r0 = threadIdx.x / kTU * RUN;
     const int u = tu * kTU + c;
-    float mm[kRun][5];
+    float mm[RUN][5];
 #pragma unroll
-    for (int o = 0; o < kRun; o++)
+    for (int o = 0; o < RUN; o++)
 #pragma unroll
         for (int k = 0; k < 5; k++) mm[o][k] = 0.f;
 #pragma unroll
-    for (int e = 0; e < 10 + kRun; e++) {
+    for (int e = 0; e < 10 + RUN; e++) {
         float x[5];
 #pragma unroll
         for (int k = 0; k < 5; k++) x[k] = h[k][r0 + e][c];
 #pragma unroll
-        for (int o = 0; o < kRun; o++) {
+        for (int o = 0; o < RUN; o++) {
             const int t = e - o;
             if (t < 0 || t > 10) continue;
 #pragma unroll
@@ -202,7 +229,7 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int 
     float S = 0.f;
     const float su = inside_mass(W, u, nu);
 #pragma unroll
-    for (int o = 0; o < kRun; o++) {
+    for (int o = 0; o < RUN; o++) {
         const int v = tv * kTV + r0 + o;
         if (u >= nu || v >= nv) continue;
         const float* m = mm[o];
@@ -231,16 +258,18 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_fwd(int nu, int nv, int 
 }
 
 // Adjoint: d_pred = scale (w * G1 + 2 x w * G2 + y w * G3), scale = -weight / (P Q).
-__global__ void __launch_bounds__(kSsimThreads) k_dssim_bwd(int nu, int nv, int ntu, const float* __restrict__ X,
+template <int RUN>
+__global__ void __launch_bounds__(Ssim<RUN>::THREADS) k_dssim_bwd(int nu, int nv, int ntu, const float* __restrict__ X,
                                                            const float* __restrict__ Y, const float* __restrict__ G,
                                                            const Window W, float scale, float* d_pred,
                                                            int accumulate) {
+    constexpr int kTV = Ssim<RUN>::TV, kInV = Ssim<RUN>::IN_V, NT = Ssim<RUN>::THREADS;
     __shared__ __align__(16) float sg[3][kInV][kInP];
     __shared__ __align__(16) float h[3][kInV][kTU];
     const int p = blockIdx.y, tu = blockIdx.x % ntu, tv = blockIdx.x / ntu;
     const int u0 = tu * kTU - kHW, v0 = tv * kTV - kHW;
     const int64_t Q = (int64_t)nu * nv, PQ = Q * gridDim.y;
-    for_staged([&](int r, int c) {
+    for_staged<RUN>([&](int r, int c) {
         const int u = u0 + c, v = v0 + r;
         const bool in = c < kInU && u >= 0 && u < nu && v >= 0 && v < nv;
         const int64_t q = (int64_t)p * Q + (int64_t)v * nu + u;
@@ -248,31 +277,31 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_bwd(int nu, int nv, int 
         for (int k = 0; k < 3; k++) sg[k][r][c] = in ? __ldg(G + k * PQ + q) : 0.f;
     });
     __syncthreads();
-    for (int i = threadIdx.x; i < kInV * (kTU / kRun); i += kSsimThreads) {
-        const int r = i / (kTU / kRun), c = (i - r * (kTU / kRun)) * kRun;
+    for (int i = threadIdx.x; i < kInV * (kTU / RUN); i += NT) {
+        const int r = i / (kTU / RUN), c = (i - r * (kTU / RUN)) * RUN;
 #pragma unroll
         for (int k = 0; k < 3; k++) {
-            float x[16], a[kRun] = {0.f, 0.f, 0.f, 0.f};
-            load16(&sg[k][r][c], x);
+            float x[16], a[RUN] = {};
+            load_staged<RUN>(&sg[k][r][c], x);
 #pragma unroll
             for (int t = 0; t < 11; t++)
 #pragma unroll
-                for (int o = 0; o < kRun; o++) a[o] = fmaf(W.w[t], x[t + o], a[o]);
-            *reinterpret_cast<float4*>(&h[k][r][c]) = make_float4(a[0], a[1], a[2], a[3]);
+                for (int o = 0; o < RUN; o++) a[o] = fmaf(W.w[t], x[t + o], a[o]);
+            store_run<RUN>(&h[k][r][c], a);
         }
     }
     __syncthreads();
-    const int c = threadIdx.x % kTU, r0 = threadIdx.x / kTU * kRun;
+    const int c = threadIdx.x % kTU, r0 = threadIdx.x / kTU * RUN;
     const int u = tu * kTU + c;
     if (u >= nu) return;
-    float bb[kRun][3];
+    float bb[RUN][3];
 #pragma unroll
-    for (int o = 0; o < kRun; o++) bb[o][0] = bb[o][1] = bb[o][2] = 0.f;
+    for (int o = 0; o < RUN; o++) bb[o][0] = bb[o][1] = bb[o][2] = 0.f;
 #pragma unroll
-    for (int e = 0; e < 10 + kRun; e++) {
+    for (int e = 0; e < 10 + RUN; e++) {
         const float x[3] = {h[0][r0 + e][c], h[1][r0 + e][c], h[2][r0 + e][c]};
 #pragma unroll
-        for (int o = 0; o < kRun; o++) {
+        for (int o = 0; o < RUN; o++) {
             const int t = e - o;
             if (t < 0 || t > 10) continue;
 #pragma unroll
@@ -280,7 +309,7 @@ __global__ void __launch_bounds__(kSsimThreads) k_dssim_bwd(int nu, int nv, int 
         }
     }
 #pragma unroll
-    for (int o = 0; o < kRun; o++) {
+    for (int o = 0; o < RUN; o++) {
         const int v = tv * kTV + r0 + o;
         if (v >= nv) break;
         const int64_t q = (int64_t)p * Q + (int64_t)v * nu + u;
@@ -497,7 +526,26 @@ __global__ void __launch_bounds__(256) k_norm_grad(const T* __restrict__ E, int6
     }
 }
 
-int ssim_tiles(int nu, int nv) { return ((nu + kTU - 1) / kTU) * ((nv + kTV - 1) / kTV); }
+// Below 200,000 pixels latency decides, and the form with four times the threads,
+// one output each on tiles half as high, is faster (both passes and the sum,
+// replayed): 16 x 16 pixels 8.4 us against 13.0, one projection of 200 x 150 10.0 and
+// 18.0, one of 512 x 384 (197,000) 18.2 and 18.8, eight of 200 x 150 (240,000) 22.1
+// and 20.3.
+bool ssim_small(int P, int nu, int nv) { return (int64_t)P * nu * nv < 200000; }
+
+int ssim_tiles(int P, int nu, int nv) {
+    const int tv = ssim_small(P, nu, nv) ? Ssim<1>::TV : Ssim<4>::TV;
+    return ((nu + kTU - 1) / kTU) * ((nv + tv - 1) / tv);
+}
+
+template <int RUN>
+void launch_dssim(int P, int nu, int nv, int nt, const float* pred, const float* meas, float C1, float C2, const Window& W,
+                  float* G, double* part, float scale, float* d_pred, int accumulate, cudaStream_t s) {
+    const int ntu = (nu + kTU - 1) / kTU;
+    const dim3 grid((unsigned)nt, (unsigned)P);
+    k_dssim_fwd<RUN><<<grid, Ssim<RUN>::THREADS, 0, s>>>(nu, nv, ntu, pred, meas, C1, C2, W, G, part);
+    if (d_pred) k_dssim_bwd<RUN><<<grid, Ssim<RUN>::THREADS, 0, s>>>(nu, nv, ntu, pred, meas, G, W, scale, d_pred, accumulate);
+}
 
 // ------------------------------------------ L1 / L2 projection loss (Eq. 10/12, Eq. 1)
 
@@ -588,7 +636,7 @@ extern "C" {
 pmf_status projection_dssim_workspace(int32_t P, int32_t nu, int32_t nv, size_t* bytes) {
     PMF_REQUIRE(bytes != nullptr && P >= 0 && nu >= 0 && nv >= 0, "bad arguments");
     *bytes = align_up(sizeof(float) * 3 * (size_t)P * nu * nv) +
-             align_up(sizeof(double) * (size_t)P * ssim_tiles(nu, nv));
+             align_up(sizeof(double) * (size_t)P * ssim_tiles(P, nu, nv));
     return PMF_OK;
 }
 
@@ -608,15 +656,12 @@ pmf_status projection_dssim(int32_t P, int32_t nu, int32_t nv, const float* pred
     double* part = (double*)((char*)ws + align_up(sizeof(float) * 3 * (size_t)P * nu * nv));
     const Window W = make_window();
     const float C1 = (0.01f * data_range) * (0.01f * data_range), C2 = (0.03f * data_range) * (0.03f * data_range);
-    const int ntu = (nu + kTU - 1) / kTU, nt = ssim_tiles(nu, nv);
+    const int nt = ssim_tiles(P, nu, nv);
+    const float scale = -weight / ((float)P * (float)nu * (float)nv);
     cudaStream_t s = (cudaStream_t)stream;
-    k_dssim_fwd<<<dim3((unsigned)nt, (unsigned)P), kSsimThreads, 0, s>>>(nu, nv, ntu, pred, meas, C1, C2, W, G, part);
-    if (d_pred) {
-        const float scale = -weight / ((float)P * (float)nu * (float)nv);
-        k_dssim_bwd<<<dim3((unsigned)nt, (unsigned)P), kSsimThreads, 0, s>>>(nu, nv, ntu, pred, meas, G, W, scale,
-                                                                          d_pred, accumulate);
-    }
-    k_dssim_final<<<1, 1024, 0, s>>>(part, nt * P, (double)P * nu * nv, weight, loss, accumulate);
+    if (ssim_small(P, nu, nv)) launch_dssim<1>(P, nu, nv, nt, pred, meas, C1, C2, W, G, part, scale, d_pred, accumulate, s);
+    else launch_dssim<4>(P, nu, nv, nt, pred, meas, C1, C2, W, G, part, scale, d_pred, accumulate, s);
+    k_dssim_final<<<1, (int64_t)nt * P <= 1024 ? 256 : 1024, 0, s>>>(part, nt * P, (double)P * nu * nv, weight, loss, accumulate);
     return check_launch("projection_dssim");
 }
 

@@ -123,3 +123,16 @@ def test_mbc_normality_of_odd_components(n, dt, offset):
     pmf.mbc_normality(g, Ed, loss=loss, d_mbc=d, accumulate=True)
     assert float(loss.item()) == pytest.approx(2.0 * ref, rel=1e-5)
     assert rel_l2(host(d), 0.5 + gref) <= 1e-6
+
+
+@pytest.mark.parametrize("shape", [(9, 177, 193), (2, 320, 320), (3, 337, 299), (1, 401, 499)])
+def test_dssim_of_many_pixels_at_tile_edges(shape):
+    """From 200,000 pixels on the four-output form: whole and ragged tiles both
+    ways, the bounds of the comparison above."""
+    P, nv, nu = shape
+    assert P * nv * nu >= 200000
+    Y, M = _projection_pair(P, nv, nu, 23)
+    loss, g = pmf.projection_dssim(dev(Y), dev(M), 300.0)
+    ref, gref = oracle.dssim(Y, M, 300.0)
+    assert abs(float(loss.item()) - ref) <= 2e-6
+    assert rel_l2(host(g), gref) <= 1e-4

@@ -813,3 +813,55 @@ def test_marchers_take_steps_beyond_their_float_cells(n):
     assert torch.equal(bt[0], gb)
     refb = oracle.project_backward(grid, 16, 16, 1.0, inside, host(dY))
     assert rel_l2(host(bt[1]), refb) <= TOL32
+
+
+def _flat_gaussians(rng, G, ratio, needles):
+    """Rotated discs or needles of the axis ratio about a small grid's centre, half
+    of them centred on voxel centres (which a flat one's ellipsoid else mostly
+    misses)."""
+    wide = np.exp(rng.uniform(np.log(3.0), np.log(8.0), G))
+    thin = wide / ratio
+    scale = np.stack([wide, thin if needles else wide * rng.uniform(0.6, 1.0, G), thin], 1).astype(np.float32)
+    mean = rng.uniform(-16.0, 16.0, (G, 3))
+    mean[::2] = 2.0 * np.round(mean[::2] / 2.0) + 1.0
+    return mean.astype(np.float32), scale, rng.normal(size=(G, 4)).astype(np.float32), \
+        rng.uniform(0.5, 1.0, (G, 1)).astype(np.float32)
+
+
+@pytest.mark.parametrize("kappa", [3.0, float("inf")])
+@pytest.mark.parametrize("needles", [False, True])
+@pytest.mark.parametrize("ratio", [30.0, 100.0, 300.0])
+def test_voxelize_keeps_flat_rotated_gaussians(ratio, needles, kappa):
+    """The render drops sub-blocks that an ellipsoid cannot reach; a flat one's
+    fp32 quadratic form loses digits to cancellation, which the drop must allow
+    for.  With u = 2^-24, R's elements are good to 20 u (a normalised quaternion's
+    products), so A's to sum_k (20 u (|R_ik| + |R_jk|) + 400 u^2 + 8 u |R_ik R_jk|) / s_k^2,
+    and q is within that times |d_i d_j|, and 8 u more of its terms, of the exact
+    one.  Every voxel lies between the sums with q that much larger and smaller,
+    give or take the terms' 2^-21 rounding and fp32's; on every tile and without a
+    list."""
+    grid, G = Grid(20, 18, 16, 2.0, 2.0, 2.0), 60
+    mean, scale, quat, value = _flat_gaussians(np.random.default_rng(int(ratio) + needles), G, ratio, needles)
+    g = pmf.Gaussians(dev(mean), dev(scale), dev(quat), dev(value), kappa)
+    got = pmf.gs_voxelize(grid, g)
+    for tile in ((16, 8, 8), (8, 8, 4), (16, 8, 4)):
+        assert torch.equal(got, pmf.gs_voxelize_tiled(grid, g, tile))
+    assert torch.equal(got, pmf.gs_voxelize(grid, g, pair_capacity=0))
+    u, ax = 2.0 ** -24, [(np.arange(n) + 0.5 - 0.5 * n) * 2.0 for n in (20, 18, 16)]
+    X = np.stack(np.meshgrid(*ax, indexing="ij"), -1).transpose(2, 1, 0, 3)  # [nz, ny, nx, 3]
+    lower, upper, k2 = 0.0, 0.0, kappa * kappa
+    for m, s, q, v in zip(mean.astype(float), scale.astype(float), quat.astype(float), value[:, 0].astype(float)):
+        w, x, y, z = q / np.linalg.norm(q)
+        R = np.array([[1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y)],
+                      [2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x)],
+                      [2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)]])
+        a = np.abs(R)
+        M = (a / s ** 2) @ a.T
+        E = 20 * u * ((a / s ** 2).sum(1)[:, None] + (a / s ** 2).sum(1)[None]) + 400 * u * u * (1 / s ** 2).sum() + 16 * u * M
+        d = X - m
+        qf = np.einsum("...i,ij,...j->...", d, (R / s ** 2) @ R.T, d)
+        dq = np.einsum("...i,ij,...j->...", np.abs(d), E, np.abs(d))
+        lower = lower + v * np.where(qf + dq <= k2, np.exp(-0.5 * (qf + dq)), 0.0)
+        upper = upper + v * np.where(qf - dq <= k2, np.exp(-0.5 * np.maximum(qf - dq, 0.0)), 0.0)
+    got, tol = host(got)[0], G * 2.0 ** -21 + 1e-6 * upper
+    assert lower.sum() > 5.0 and np.all(got >= lower - tol) and np.all(got <= upper + tol)

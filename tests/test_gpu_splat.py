@@ -177,3 +177,42 @@ def test_rasterize_adjoint_run_blocks(nu):
     ref = oracle.splat_backward(det.nu, det.nv, vw, gs.mean, gs.scale, gs.quat, gs.value, dY, 3.0)
     for name, a, b in zip(("mean", "scale", "quat", "value"), got, ref):
         assert rel_l2(host(a), np.asarray(b).reshape(tuple(a.shape))) <= TOLG, name
+
+
+@pytest.mark.parametrize("kappa", [3.0, float("inf")])
+@pytest.mark.parametrize("ratio", [10.0, 30.0, 100.0])
+def test_rasterize_keeps_flat_rotated_gaussians(ratio, kappa):
+    """The render drops pixel blocks that a projected ellipse cannot reach; a flat
+    one's fp32 quadratic form loses digits, which the drop must allow for.  With
+    u = 2^-24 the elements of Sigma^ are good to 30 u of its largest (three-term
+    sums of products good to 10 u), so the form and its inverse to 100 u cond q;
+    p^ to an ulp adds 2 |K d| of it.  Every pixel lies between the sums with q
+    that much larger and smaller, and rho^ a thousandth (40 u ratio, at most
+    2.4e-4), give or take the pixel sums' 2^-21 rounding; with and without lists."""
+    rng = np.random.default_rng(62 + int(ratio))
+    G, nu, nv = 60, 40, 29
+    wide = np.exp(rng.uniform(np.log(4.0), np.log(14.0), G))
+    scale = np.stack([wide, np.where(np.arange(G) % 2, wide / ratio, wide), wide / ratio], 1).astype(np.float32)
+    mean, quat = rng.uniform(-12.0, 12.0, (G, 3)).astype(np.float32), rng.normal(size=(G, 4)).astype(np.float32)
+    value = rng.uniform(0.5, 1.0, (G, 1)).astype(np.float32)
+    vw, det = circular_views(2, 300.0, 450.0, nu, nv, 1.4, 1.4, start=0.4), Detector(nu, nv, 1.0)
+    g = pmf.Gaussians(dev(mean), dev(scale), dev(quat), dev(value), kappa)
+    got = pmf.gs_rasterize(det, views(vw), g)
+    assert torch.equal(got, pmf.gs_rasterize(det, views(vw), g, pair_capacity=1))
+    xa, xb = np.meshgrid(np.arange(nu) + 0.5 - nu / 2, np.arange(nv) + 0.5 - nv / 2)
+    u, k2 = 2.0 ** -24, kappa * kappa
+    for p in range(2):
+        lower, upper, top = np.zeros((nv, nu)), np.zeros((nv, nu)), 0.0
+        for i in range(G):
+            pa, pb, s00, s01, s11, rho = oracle.splat_params(vw[p], mean[i], scale[i], quat[i], value[i, 0])[:6]
+            S = np.array([[s00, s01], [s01, s11]])
+            K, ev = np.linalg.inv(S), np.linalg.eigvalsh(S)
+            d = np.stack([xa - pa, xb - pb], -1)
+            Kd = d @ K
+            q = (Kd * d).sum(-1)
+            dq = 100 * u * ev[1] / ev[0] * q + 2 * np.linalg.norm(Kd, axis=-1) * 2 * u * (abs(pa) + abs(pb) + nu)
+            lower += 0.999 * rho * np.where(q + dq <= k2, np.exp(-0.5 * (q + dq)), 0.0)
+            upper += 1.001 * rho * np.where(q - dq <= k2, np.exp(-0.5 * np.maximum(q - dq, 0.0)), 0.0)
+            top = max(top, rho)
+        y, tol = host(got)[p], top * G * 2.0 ** -21 + 1e-6 * upper
+        assert lower.sum() > 10.0 and np.all(y >= lower - tol) and np.all(y <= upper + tol)
