@@ -214,8 +214,10 @@ __device__ __forceinline__ void gather_global(const T* __restrict__ V, const Gri
 }
 
 // One 16 x (RPB/16) pixel tile of view p: every thread of the CTA calls it.  Not
-// STAGED: every chunk is gathered (plain_exact).
-template <typename T, int CH, int RPB, bool STAGED>
+// STAGED: every chunk is gathered (plain_exact).  PAIRS: gathered by pairs; the
+// batched kernels, whose item leaves fewer registers, spill with them (four odd
+// fp32 volumes 1,325 -> 1,423 us with hardly a chunk gathered) and go one by one.
+template <typename T, int CH, int RPB, bool STAGED, bool PAIRS>
 __device__ __forceinline__ void project_tile(const GridD& g, int nu, int nv, int ntu, float step,
                                              const pmf_view* __restrict__ views, const T* __restrict__ vol,
                                              int64_t vol_stride, float* __restrict__ proj, int p, int tile,
@@ -256,7 +258,12 @@ __device__ __forceinline__ void project_tile(const GridD& g, int nu, int nv, int
                 else gather_samples<65, kPlainBox, false>(r, box, q0, sz, j0, j1, fb, acc);
             }
         } else if (act) {
-            gather_global(V, g, r, ib, fb, j0, j1, acc);
+            if constexpr (PAIRS) {
+                gather_global(V, g, r, ib, fb, j0, j1, acc);
+            } else {
+                float jf = (float)j0;
+                for (int j = j0; j <= j1; j++, jf += 1.0f) acc += gather_one(V, g, r, ib, fb, jf);
+            }
         }
         __syncthreads();
     }
@@ -269,7 +276,7 @@ __global__ void __launch_bounds__(RPB, 1024 / RPB) k_project(GridD g, int nu, in
                                                   int64_t vol_stride, float* __restrict__ proj) {
     extern __shared__ __align__(128) float box[];  // kPlainBox floats
     __shared__ BoxState bs;
-    project_tile<T, CH, RPB, STAGED>(g, nu, nv, ntu, step, views, vol, vol_stride, proj, blockIdx.y, blockIdx.x, box, bs);
+    project_tile<T, CH, RPB, STAGED, true>(g, nu, nv, ntu, step, views, vol, vol_stride, proj, blockIdx.y, blockIdx.x, box, bs);
 }
 
 // ------------------------------------------- forward with bulk-copy staging
@@ -499,7 +506,7 @@ __global__ void __launch_bounds__(RPB, 1024 / RPB) k_project_batched(const __gri
     for (int64_t w = blockIdx.x; w < B.total; w += gridDim.x) {
         const ProjItem it = B.it[find_item(B, w)];  // a copy: the tile code reads registers, not the parameter block
         const int local = (int)(w - it.begin);  // < 2^31: checked when the item is filled
-        project_tile<T, CH, RPB, STAGED>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, (const T*)it.vol, it.vol_stride, it.proj,
+        project_tile<T, CH, RPB, STAGED, false>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, (const T*)it.vol, it.vol_stride, it.proj,
                         local / it.ntiles, local % it.ntiles, box, bs);
         __syncthreads();
     }
@@ -533,7 +540,7 @@ __global__ void __launch_bounds__(RPB, 1024 / RPB) k_project_batched1(const __gr
     const int64_t w = blockIdx.x;
     const ProjItem it = B.it[find_item(B, w)];
     const int local = (int)(w - it.begin);
-    project_tile<T, CH, RPB, true>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, (const T*)it.vol, it.vol_stride, it.proj,
+    project_tile<T, CH, RPB, true, false>(it.g, it.nu, it.nv, it.ntu, it.step, it.views, (const T*)it.vol, it.vol_stride, it.proj,
                     local / it.ntiles, local % it.ntiles, box, bs);
 }
 
