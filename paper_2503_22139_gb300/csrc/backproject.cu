@@ -161,8 +161,8 @@ __device__ __forceinline__ int exp_for(float bound, int bits) {
 // atomic whose 32 addresses lie in distinct banks takes one wavefront
 // (measured); each further address in the busiest bank adds one.  This layout
 // spreads the 32 simultaneous corner addresses over the banks (measured at the
-// paper geometry: 2.85 wavefronts per warp-wide atomic with the ray-following
-// box layout below, 3.8 with a fixed one).
+// paper geometry with 32-sample chunks: 2.85 wavefronts per warp-wide atomic with
+// the ray-following box layout below, 3.8 with a fixed one; 2.64 with 48).
 template <int RPB>
 __device__ __forceinline__ void pixel_of_spread(int tile, int ntu, int& a, int& b) {
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, g = l & 7, q = l >> 3;

@@ -27,7 +27,7 @@ namespace {
 
 // Launch shapes (MarchShape): CH samples per chunk (the staged brick's length
 // along the rays) and RPB rays per CTA (a 16 x RPB/16 pixel tile, one ray per
-// thread).  The C entry points use 32 and 256 for the projector, 48 and 128
+// thread).  The C entry points use 48 and 256 for the projector, 48 and 128
 // for the adjoint; plans may pick others.
 constexpr unsigned kFull = 0xffffffffu;
 

@@ -260,9 +260,10 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
 
 // Floors without the conversion pipe: adding 1.5 2^23 rounded down leaves
 // floor(u) in the low bits of the sum, exact for |u| < 2^22, and the sum less
-// 1.5 2^23 is the floor as a float.  The ray marcher's adjoint takes it (1,830 ->
-// 1,802 us for 8 views at the paper geometry); the projector, whose fp32 pipe
-// has less to spare, takes it for one of the three axes (4% slower with all).
+// 1.5 2^23 is the floor as a float.  The ray marcher's adjoint takes it in place of
+// conversions (as fast as with them: 1,801 and 1,828 us for 8 views at the paper
+// geometry, runs of one form differing by 3%); the projector, whose fp32 pipe has
+// less to spare, takes it for one of the three axes (4% slower with all).
 constexpr float kFloorBias = 12582912.0f;
 constexpr unsigned kFloorBits = 0x4b400000u;  // its bit pattern
 

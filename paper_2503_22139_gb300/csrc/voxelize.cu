@@ -7,10 +7,10 @@
 // tile stages its list in shared memory and sums every entry at its 512 voxel
 // centres.  Sums are exact integers at the scale 2^k with max|value| 2^k < 2^21:
 // each term is rounded once to an integer (magic-number add), a batch of at
-// most 256 terms is summed in 32 bits (< 2^29) and batches are added in 64
+// most 512 terms is summed in 32 bits (< 2^30) and batches are added in 64
 // bits, so the unordered list fill cannot change a bit of the result.
 //
-// Backward: one CTA per Gaussian walks its voxel box, accumulates
+// Backward: one warp per Gaussian and slab of its voxel box's rows accumulates
 // sum_v dL/dout_c * e, and the moments S1 = sum w d, S2 = sum w d d^T
 // (w = e * sum_c value_c dL/dout_c), reduces them in a fixed order, and turns
 // them into d mean = A S1, d scale_j = (R^T S2 R)_jj / s_j^3,

@@ -45,14 +45,16 @@ def _shape(g):
     return (gr.nz, gr.ny, gr.nx), gr.nx * gr.ny * gr.nz
 
 
+# The current stream's handle itself (building a torch.cuda.Stream around it takes
+# about 10 us of each call), where torch has the call for it, which is not part of
+# its public interface.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream():
-    # the current stream's handle itself (building a torch.cuda.Stream around it
-    # takes about 10 us of each call) where torch has the call for it, which is
-    # not part of its public interface
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    if raw is None:
+    if _raw_stream is None:
         return ct.c_void_p(torch.cuda.current_stream().cuda_stream)
-    return ct.c_void_p(raw(torch.cuda.current_device()))
+    return ct.c_void_p(_raw_stream(torch.cuda.current_device()))
 
 
 def _p(t: Optional[torch.Tensor]):

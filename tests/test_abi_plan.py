@@ -190,6 +190,6 @@ def test_pair_capacity_refuses_unsupported_tiles(tile):
 def test_stream_handle_without_the_private_torch_call(monkeypatch):
     """torch's raw-stream call is not public: without it the handle comes from
     the current stream's object."""
-    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(ops, "_raw_stream", None)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0x1234))
     assert ops._stream().value == 0x1234
