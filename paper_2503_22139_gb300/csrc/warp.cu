@@ -142,24 +142,23 @@ bool runs_aligned(int64_t N, const void* a, const void* b) {
     return N % V == 0 && ((((uintptr_t)a) | ((uintptr_t)b)) & 15) == 0;
 }
 
-// Streams E once and D once per view, LL levels (0: the runtime L) of V
-// consecutive voxels in registers.  Bandwidth bound: at the paper grid, three
-// levels and one fp32 view, 192 MB take 28 us at the copy rate; one voxel per
-// thread with the level count at run time took 60 us, four per thread 27.
-template <typename T, int LL, int V>
-__global__ void __launch_bounds__(kThreads) k_combine(GridD g, int Lr, int P, const T* __restrict__ E,
+// Streams E once and D once per view, L levels of V consecutive voxels in
+// registers.  Bandwidth bound: at the paper grid, three levels and one fp32
+// view, 192 MB take 28 us at the copy rate; one voxel per thread with the level
+// count at run time took 60 us, four per thread 27.  Every count is a template
+// argument: eight bf16 levels, one view, one voxel per thread took 121 us with
+// the count at run time, 139 with the loops over all eight tested for it, 43 so.
+template <typename T, int L, int V>
+__global__ void __launch_bounds__(kThreads) k_combine(GridD g, int P, const T* __restrict__ E,
                                                       const float* __restrict__ w, T* __restrict__ D) {
-    constexpr int M = LL ? LL : kMaxL;
-    const int L = LL ? LL : Lr;
     const int64_t N = g.n;
     for (int64_t v = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); v < N;
          v += V * (int64_t)gridDim.x * blockDim.x) {
-        float e[M][3][V];
+        float e[L][3][V];
 #pragma unroll
-        for (int l = 0; l < M; l++)
+        for (int l = 0; l < L; l++)
 #pragma unroll
-            for (int k = 0; k < 3; k++)
-                if (l < L) ld_run<V>(E + ((int64_t)l * 3 + k) * N + v, e[l][k]);
+            for (int k = 0; k < 3; k++) ld_run<V>(E + ((int64_t)l * 3 + k) * N + v, e[l][k]);
         for (int p = 0; p < P; p++) {
 #pragma unroll
             for (int k = 0; k < 3; k++) {
@@ -167,12 +166,11 @@ __global__ void __launch_bounds__(kThreads) k_combine(GridD g, int Lr, int P, co
 #pragma unroll
                 for (int i = 0; i < V; i++) acc[i] = 0.f;
 #pragma unroll
-                for (int l = 0; l < M; l++)
-                    if (l < L) {
-                        const float c = __ldg(w + (p * L + l) * 3 + k);
+                for (int l = 0; l < L; l++) {
+                    const float c = __ldg(w + (p * L + l) * 3 + k);
 #pragma unroll
-                        for (int i = 0; i < V; i++) acc[i] = fmaf(c, e[l][k][i], acc[i]);
-                    }
+                    for (int i = 0; i < V; i++) acc[i] = fmaf(c, e[l][k][i], acc[i]);
+                }
                 st_run<V>(D + ((int64_t)p * 3 + k) * N + v, acc);
             }
         }
@@ -1146,16 +1144,15 @@ void launch_combine(const GridD& g, int L, int P, const void* mbc, const float* 
     T* D = (T*)dvf;
     const bool run4 = runs_aligned<4>(g.n, mbc, dvf);
     const unsigned nb = stream_blocks(run4 ? (g.n + 3) / 4 : g.n);
-#define PMF_COMBINE(LL)                                                                       \
-    if (run4) k_combine<T, LL, 4><<<nb, kThreads, 0, s>>>(g, L, P, E, coeff, D);              \
-    else k_combine<T, LL, 1><<<nb, kThreads, 0, s>>>(g, L, P, E, coeff, D);                   \
-    break;
+#define PMF_COMBINE(L_)                                                                   \
+    case L_:                                                                              \
+        if (run4) k_combine<T, L_, 4><<<nb, kThreads, 0, s>>>(g, P, E, coeff, D);         \
+        else k_combine<T, L_, 1><<<nb, kThreads, 0, s>>>(g, P, E, coeff, D);              \
+        break;
+    static_assert(kMaxL == 8, "a case per level count");
     switch (L) {
-        case 1: PMF_COMBINE(1)
-        case 2: PMF_COMBINE(2)
-        case 3: PMF_COMBINE(3)
-        case 4: PMF_COMBINE(4)
-        default: k_combine<T, 0, 1><<<stream_blocks(g.n), kThreads, 0, s>>>(g, L, P, E, coeff, D);
+        PMF_COMBINE(1) PMF_COMBINE(2) PMF_COMBINE(3) PMF_COMBINE(4)
+        PMF_COMBINE(5) PMF_COMBINE(6) PMF_COMBINE(7) PMF_COMBINE(8)
     }
 #undef PMF_COMBINE
 }

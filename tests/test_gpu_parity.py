@@ -865,3 +865,19 @@ def test_voxelize_keeps_flat_rotated_gaussians(ratio, needles, kappa):
         upper = upper + v * np.where(qf - dq <= k2, np.exp(-0.5 * np.maximum(qf - dq, 0.0)), 0.0)
     got, tol = host(got)[0], G * 2.0 ** -21 + 1e-6 * upper
     assert lower.sum() > 5.0 and np.all(got >= lower - tol) and np.all(got <= upper + tol)
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("L", [5, 6, 7, 8])
+def test_combine_levels_above_four(L, dt):
+    """mbc_combine at five to eight levels, in runs of four voxels and one by one
+    (an odd voxel count): the sum in 32 bits over the stored vectors, rounded once."""
+    tol = {torch.float32: TOL32, torch.bfloat16: 2.0**-8, torch.float16: 2.0**-11}[dt]
+    for n, P in (((12, 6, 5), 3), ((11, 7, 5), 1), ((67, 66, 64), 2)):
+        grid = Grid(*n, 2.0, 2.0, 2.0)
+        rng = np.random.default_rng(490 + L)
+        E = dev(rng.normal(size=(L, 3) + grid.shape).astype(np.float32)).to(dt)
+        w = rng.normal(size=(P, L, 3)).astype(np.float32)
+        got = pmf.mbc_combine(grid, E, dev(w))
+        ref = np.einsum("plk,lkzyx->pkzyx", w.astype(np.float64), E.double().cpu().numpy())
+        assert got.dtype == dt and rel_l2(host(got.float()), ref) <= tol
