@@ -1334,10 +1334,36 @@ pmf_status warp_volume_backward(const pmf_grid* grid, int32_t P, pmf_dtype dtype
 namespace pmf {
 namespace {
 
+// CTAs of the tiled forward per SM, held down by the shared memory asked for.
+// Where tiles end inside a 32-byte sector (fp32 rows not a multiple of four
+// voxels), neighbouring CTAs complete each other's sectors in L2, and with too
+// many views in flight (CTAs x views x a tile's 1 KB) lines leave it half
+// written: beyond 40 views or so each further one costs twice.  Fewer CTAs move
+// that edge up, at 5 to 7% a CTA below it; it comes later with more levels, and
+// later in even rows.  201 x 199 x 99 voxels, six, five, four CTAs: one level 48
+// views 453, 378, 406 us, 96 views 1,050, 900, 792; two levels 64 views 608-635,
+// 514, 546, 96 views 1,045, 888, 783; three levels 48 views 414, 442, 473, 64 views
+// 580-607, 565, 596.  202 x 200 x 100: one level 48 views 401, 373, 404; two levels
+// 64 views 479-524, 508, 543, 96 views 908-937, 727, 775; three levels 96 views 774,
+// 793, 840, 128 views 1,212, 1,034, 1,091.  One level at 32 views: 299 -> 273, 203 x
+// 161 x 87 209 -> 203.  Rows of 204 or 200 voxels, 16-bit outputs, and outputs that L2
+// holds (65 x 64 x 64, 48 views) have no such edge.
+size_t wc_fwd_smem(const GridD& g, int L, int P, size_t out_size) {
+    constexpr size_t kSmSmem = 228 * 1024, kReserved = 1024;
+    const size_t need = sizeof(float4) * (size_t)(P * L) + sizeof(float2) * (size_t)GeomFwd::BOXN;
+    const bool odd = g.nx % 2 != 0;
+    if (out_size < 4 || g.nx % 4 == 0 || P < 16 + (odd ? 16 : 32) * L) return need;
+    if (g.n * P * (int64_t)out_size < (64 << 20)) return need;
+    const size_t ctas = odd && P >= 96 ? 4 : 5;
+    const size_t hold = kSmSmem / (ctas + 1) - kReserved + 128;  // one more CTA does not fit
+    return need > hold ? need : hold;
+}
+static_assert(sizeof(float4) * kMaxPLTile + sizeof(float2) * GeomFwd::BOXN <= 48 * 1024 && 228 * 1024 / 5 <= 48 * 1024,
+              "the forward's shared memory needs no larger limit set");
+
 template <typename T, typename TO, int LL>
 void launch_wc_fwd(unsigned nt, size_t smem, cudaStream_t s, const GridD& g, int P, const void* ref, const void* mbc,
                    const float* coeff, void* out) {
-    cudaFuncSetAttribute(k_wc_fwd_tile<T, TO, LL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_wc_fwd_tile<T, TO, LL><<<nt, GeomFwd::THREADS, smem, s>>>(g, P, (const T*)ref, (const T*)mbc, coeff, (TO*)out);
 }
 
@@ -1345,7 +1371,7 @@ template <typename T, typename TO>
 pmf_status launch_warp_combine(const GridD& g, int32_t L, int32_t P, const void* ref, const void* mbc,
                                const float* coeff, void* out, cudaStream_t s) {
     if (L <= 4 && (int64_t)P * L <= kMaxPLTile && g.n < ((int64_t)1 << 31)) {
-        const size_t smem = sizeof(float4) * (size_t)(P * L) + sizeof(float2) * (size_t)GeomFwd::BOXN;
+        const size_t smem = wc_fwd_smem(g, L, P, sizeof(TO));
         const unsigned nt = (unsigned)num_tiles<GeomFwd>(g);
         switch (L) {
             case 1: launch_wc_fwd<T, TO, 1>(nt, smem, s, g, P, ref, mbc, coeff, out); break;

@@ -881,3 +881,19 @@ def test_combine_levels_above_four(L, dt):
         got = pmf.mbc_combine(grid, E, dev(w))
         ref = np.einsum("plk,lkzyx->pkzyx", w.astype(np.float64), E.double().cpu().numpy())
         assert got.dtype == dt and rel_l2(host(got.float()), ref) <= tol
+
+
+@pytest.mark.parametrize("nx,L,P", [(33, 1, 31), (33, 1, 32), (33, 2, 48), (33, 3, 64), (33, 4, 80), (33, 1, 95),
+                                    (33, 1, 96), (33, 4, 128), (34, 1, 48), (34, 3, 111), (34, 3, 112)])
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+def test_warp_combine_many_views_of_ragged_rows(nx, L, P, dt):
+    """The fused forward at the view counts from which fewer CTAs run per SM (fp32
+    rows not a multiple of four voxels): the same volumes as in calls of 16 views."""
+    grid = Grid(nx, 130, 131, 2.0, 2.0, 2.0)
+    V, E, w = _mbc_and_ref(grid, 500 + P, L=L, P=P)
+    Vd, Ed, wd = dev(V).to(dt), dev(E).to(dt), dev(w)
+    out = torch.full((P,) + grid.shape, float("nan"), device="cuda")
+    got = pmf.warp_combine(grid, Vd, Ed, wd, out=out)
+    for p in range(0, P, 16):
+        part = torch.empty((min(16, P - p),) + grid.shape, device="cuda")
+        assert torch.equal(got[p:p + 16], pmf.warp_combine(grid, Vd, Ed, wd[p:p + 16], out=part))
